@@ -161,6 +161,7 @@ struct ChirpParams {
     // the wrap); the output tables undo it with exp(+2 pi i k sh / nf).
     int sh1, sh2;
     double screen_k;       // 2 pi / lambda of the problem (source screens)
+    int row_base;          // added to a record's s2: problem * nf2 for strip-sorted plans, else 0
 };
 
 // Piecewise-polynomial form of the spreading kernel: the value at
@@ -278,6 +279,23 @@ struct FamTable {
 };
 constexpr int kNodeThreads = 256;
 
+// Sort of a strip-sorted plan (strips.cuh): every record once, under the key
+// of its first support cell: 128 keys per live 32 x 32 tile (live[tile]: its
+// index, -1 for tiles that no support touches), 8-column strip by row.
+constexpr int kStripKeys = 4 * kTile;   // keys per live tile
+struct StripSort {
+    const int* live;    // per tile of every problem
+    int* counts;        // records per key (zero between evaluations)
+    int* start;         // first sorted position per key
+    int* rank;          // per record: its place within its key
+    int* cursor;        // places handed out so far (zero between evaluations)
+    int nkeys;
+    int ntx;
+};
+__host__ __device__ __forceinline__ int strip_key(int live, int s1, int s2) {
+    return live * kStripKeys + ((s1 & (kTile - 1)) >> 3) * kTile + (s2 & (kTile - 1));
+}
+
 // Per-problem regions of a batched plan's chunk list, split-tile list and
 // sorted records (B + 1 entries each, absolute starts; sized at plan time).
 // Chunk index space: every problem's split chunks first, then every
@@ -307,6 +325,15 @@ void launch_nodes(const FamTable& ft, int nblocks, NodeRec<T>* rec, int* counts,
 template <typename T>
 void launch_scatter_fams(const FamTable& ft, int nblocks, const NodeRec<T>* rec, int* cursor,
                          NodeRec<T>* sorted, long long cap, unsigned* status, cudaStream_t st);
+// Strip-sorted plans: the node pass (records, key counts and ranks), then key
+// starts and the scatter of the n records.
+template <typename T>
+void launch_nodes_strips(const FamTable& ft, int nblocks, NodeRec<T>* rec, const StripSort& ss,
+                         double* dx, double* dy, double* dw, unsigned* status, cudaStream_t st);
+void launch_strip_starts(const StripSort& ss, cudaStream_t st);
+template <typename T>
+void launch_scatter_strips(long long n, const NodeRec<T>* rec, const StripSort& ss,
+                           NodeRec<T>* sorted, unsigned* status, cudaStream_t st);
 // One block per problem (B blocks): cursors, chunks and split tiles into the
 // problem's regions of L; clears the counts.
 void launch_scan_problems(int B, int ntiles, int* counts, int* cursor, Chunk* chunks,
@@ -344,6 +371,11 @@ void launch_spread(const NodeRec<T>* sorted, const Chunk* chunks, const int* n_m
                    int max_chunks, int* ready, int max_split, long long max_spin,
                    cx_t<T>* grid, int* work, unsigned* status, int nf1, int nf2, int ntx,
                    int ntiles, const KernelShape& ks, int nblocks, cudaStream_t st);
+// Strip-sorted records (strips.cuh): adds n records into the grid, which must
+// be zero; problems' grids are stacked by rows (record s2 = problem * nf2 + row).
+template <typename T>
+void launch_spread_strips(const NodeRec<T>* sorted, long long n, cx_t<T>* grid, int nf1, int nf2,
+                          const KernelShape& ks, cudaStream_t st);
 // Deterministic mode (fresnel_opts.deterministic): the same grid from exact
 // fixed-point sums, bit for bit whatever the records' order within a tile
 // and the split tiles' chunk order.  Three launches: the strengths' partial
@@ -383,7 +415,7 @@ void launch_adj_shape_reduce(const FamilyDev* fams, const int* sf, int nsf, int 
 
 // k_fft.cu
 struct RowPassArgs {
-    const void* in; void* out;
+    void* in; void* out;
     long long in_stride, out_stride;   // elements between rows
     int nrows;
     int in_len;          // input elements per row
@@ -400,9 +432,12 @@ struct RowPassArgs {
     // walking every row and skipping dead ones by their live flag
     const int* row_list;
     int nlist;
+    // 1: the nonzero inputs are set to zero once read (strip-sorted plans: the
+    // next evaluation's spread adds into a zero grid)
+    int clear_in;
 };
 struct ColPassArgs {
-    const void* in; void* out;
+    void* in; void* out;
     int ncols;           // columns (contiguous dimension length of in/out)
     int in_len;          // input rows
     int centered_in;
@@ -437,6 +472,7 @@ struct ColPassArgs {
     const void* twN;
     const void* deconv_col;
     const void* deconv_row;
+    int clear_in;        // kFftRowStep1: as RowPassArgs
 };
 enum { kFftPlain = 0, kFftRowStep1 = 1, kFftColStep1 = 2, kFftColStep2 = 3, kFftRowStep2 = 4 };
 template <typename T>

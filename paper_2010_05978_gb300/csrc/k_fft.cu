@@ -163,6 +163,20 @@ __host__ __device__ __forceinline__ int padded_len(int n) { return n + (n >> 4) 
 
 template <typename T> __host__ __device__ constexpr int emax() { return 8; }
 
+// The input side of a transform: load(e) reads natural input e, use(e, v)
+// turns the value read into the value transformed (a factor, and where asked
+// for the input set back to zero).  Apart, so that a butterfly's loads are
+// all in flight before a store that may alias them: with the zeroing inside
+// the load the 64-wavelength sweep's row pass took 35 us instead of 21.
+template <class L, class U>
+struct Input {
+    L l;
+    U u;
+    __device__ __forceinline__ auto operator()(int e) const { return l(e); }
+    template <class C> __device__ __forceinline__ C use(int e, C v) const { return u(e, v); }
+};
+template <class L, class U> __device__ __forceinline__ Input<L, U> make_input(L l, U u) { return {l, u}; }
+
 // A stage whose inputs come from global memory (FIRST: load(e) for natural
 // input index e, always p = 1) and/or whose outputs go straight to global
 // memory (LAST: store(k, value) for natural output index k); otherwise as
@@ -185,11 +199,15 @@ __device__ __forceinline__ void stage_io(const cx_t<T>* __restrict__ src, cx_t<T
 #pragma unroll
         for (int q = 0; q < R; ++q) {
             if constexpr (FIRST) {
-                u[q] = load(i + q * nb);
+                u[q] = load(i + q * nb);   // all R loads in flight before the first use
             } else {
                 u[q] = src[pad(i + q * nb) * NCOL + c];
                 if (q > 0 && k > 0) u[q] = O::mul(u[q], __ldg(&tw[q * kt]));
             }
+        }
+        if constexpr (FIRST) {
+#pragma unroll
+            for (int q = 0; q < R; ++q) u[q] = load.use(i + q * nb, u[q]);
         }
         Dft<T, R>::run(u, y);
         const int j = (i - k) * R + k;
@@ -280,16 +298,25 @@ k_fft_rows(FftPlan fp, RowPassArgs a) {
         return r;
     };
     auto transform = [&](int row) {
-        const C* in = (const C*)a.in + (long long)row * a.in_stride;
+        C* in = (C*)a.in + (long long)row * a.in_stride;
         C* out = (C*)a.out + (long long)row * a.out_stride;
         const T rowf = a.deconv_row ? ((const T*)a.deconv_row)[row] : (T)1;
-        auto load = [&](int e) {
-            const int i = in_src(e, a.in_len, n, a.centered_in);
-            if (i < 0) return Ops<T>::mk(0, 0);
-            C v = in[i];
-            if (a.centered_in) v = Ops<T>::scale(v, rowf * (dcol ? dcol[i] : (T)1));
-            return v;
-        };
+        auto load = make_input(
+            [&](int e) {
+                const int i = in_src(e, a.in_len, n, a.centered_in);
+                if (i < 0) return Ops<T>::mk(0, 0);
+                C v = in[i];
+                if (a.centered_in) {
+                    if (a.clear_in && (v.x != (T)0 || v.y != (T)0)) in[i] = Ops<T>::mk(0, 0);
+                    v = Ops<T>::scale(v, rowf * (dcol ? dcol[i] : (T)1));
+                }
+                return v;
+            },
+            [&](int e, C v) {
+                if (a.clear_in && !a.centered_in && (v.x != (T)0 || v.y != (T)0) && e < a.in_len)
+                    in[e] = Ops<T>::mk(0, 0);
+                return v;
+            });
         auto store = [&](int k, C v) {
             const int kp = out_slot(k, a.out_len, n);
             if (kp >= 0) out[kp] = v;
@@ -338,15 +365,17 @@ k_fft_cols(FftPlan fp, ColPassArgs a) {
                 axc = ((const C*)a.ax)[(long long)bi * a.ncols + col];
                 ay = (const C*)a.ay + (long long)bi * a.out_len;
             }
-            auto load = [&](int e) {
-                const int i = in_src(e, a.in_len, n, a.centered_in);
-                if (i < 0 || !on) return Ops<T>::mk(0, 0);
-                if (a.live) {
-                    const int tr = i / kTile;
-                    if (!((s_live[tr >> 5] >> (tr & 31)) & 1u)) return Ops<T>::mk(0, 0);
-                }
-                return in[(long long)i * a.ncols];
-            };
+            auto load = make_input(
+                [&](int e) {
+                    const int i = in_src(e, a.in_len, n, a.centered_in);
+                    if (i < 0 || !on) return Ops<T>::mk(0, 0);
+                    if (a.live) {
+                        const int tr = i / kTile;
+                        if (!((s_live[tr >> 5] >> (tr & 31)) & 1u)) return Ops<T>::mk(0, 0);
+                    }
+                    return in[(long long)i * a.ncols];
+                },
+                [](int, C v) { return v; });
             auto store = [&](int k, C v) {
                 const int kp = out_slot(k, a.out_len, n);
                 if (kp < 0 || !on) return;
@@ -359,18 +388,21 @@ k_fft_cols(FftPlan fp, ColPassArgs a) {
             fft_fused<T, NCOL>(S, S2, fp, tw, load, store);
         } else if constexpr (MODE == kFftRowStep1) {
             // grid row o viewed as fa x fb (element e = fb a + b at column b = col)
-            const C* in = (const C*)a.in + (long long)o * a.in_stride;
+            C* in = (C*)a.in + (long long)o * a.in_stride;
             C* out = (C*)a.out + (long long)o * a.fN + col;
             const T rowf = a.deconv_row ? ((const T*)a.deconv_row)[o] : (T)1;
             const T* dcol = (const T*)a.deconv_col;
-            auto load = [&](int ea) {
-                if (!on) return Ops<T>::mk(0, 0);
-                const int i = in_src(a.fb * ea + col, a.in_len, a.fN, a.centered_in);
-                if (i < 0) return Ops<T>::mk(0, 0);
-                C v = in[i];
-                if (a.centered_in) v = Ops<T>::scale(v, rowf * (dcol ? dcol[i] : (T)1));
-                return v;
-            };
+            auto load = make_input(
+                [&](int ea) {
+                    if (!on) return Ops<T>::mk(0, 0);
+                    const int i = in_src(a.fb * ea + col, a.in_len, a.fN, a.centered_in);
+                    if (i < 0) return Ops<T>::mk(0, 0);
+                    C v = in[i];
+                    if (a.clear_in && (v.x != (T)0 || v.y != (T)0)) in[i] = Ops<T>::mk(0, 0);
+                    if (a.centered_in) v = Ops<T>::scale(v, rowf * (dcol ? dcol[i] : (T)1));
+                    return v;
+                },
+                [](int, C v) { return v; });
             auto store = [&](int k1, C v) {
                 if (on) out[(long long)k1 * a.fb] = v;
             };
@@ -379,12 +411,13 @@ k_fft_cols(FftPlan fp, ColPassArgs a) {
             // outer index o = b: rows e = fb a + b of the grid columns
             const C* in = (const C*)a.in + col;
             C* out = (C*)a.out + (long long)o * a.ncols + col;
-            auto load = [&](int ea) {
-                if (!on) return Ops<T>::mk(0, 0);
-                const int i = in_src(a.fb * ea + o, a.in_len, a.fN, a.centered_in);
-                if (i < 0) return Ops<T>::mk(0, 0);
-                return in[(long long)i * a.ncols];
-            };
+            auto load = make_input(
+                [&](int ea) {
+                    if (!on) return Ops<T>::mk(0, 0);
+                    const int i = in_src(a.fb * ea + o, a.in_len, a.fN, a.centered_in);
+                    return i < 0 ? Ops<T>::mk(0, 0) : in[(long long)i * a.ncols];
+                },
+                [](int, C v) { return v; });
             auto store = [&](int k1, C v) {
                 if (on) out[(long long)k1 * a.fb * a.ncols] = v;
             };
@@ -394,10 +427,12 @@ k_fft_cols(FftPlan fp, ColPassArgs a) {
             const C* in = (const C*)a.in + ((long long)o * a.fa + col) * a.fb;
             C* out = (C*)a.out + (long long)o * a.out_stride;
             const C* twN = (const C*)a.twN;
-            auto load = [&](int b) {
-                if (!on) return Ops<T>::mk(0, 0);
-                return Ops<T>::mul(in[b], __ldg(&twN[b * col]));
-            };
+            auto load = make_input(
+                [&](int b) {
+                    if (!on) return Ops<T>::mk(0, 0);
+                    return Ops<T>::mul(in[b], __ldg(&twN[b * col]));
+                },
+                [](int, C v) { return v; });
             auto store = [&](int k2, C v) {
                 const int kp = out_slot(col + a.fa * k2, a.out_len, a.fN);
                 if (kp >= 0 && on) out[kp] = v;
@@ -409,10 +444,12 @@ k_fft_cols(FftPlan fp, ColPassArgs a) {
             const C* twN = (const C*)a.twN;
             C axc = Ops<T>::mk(1, 0);
             if (a.ax && on) axc = ((const C*)a.ax)[col];
-            auto load = [&](int b) {
-                if (!on) return Ops<T>::mk(0, 0);
-                return Ops<T>::mul(in[(long long)b * a.ncols], __ldg(&twN[b * o]));
-            };
+            auto load = make_input(
+                [&](int b) {
+                    if (!on) return Ops<T>::mk(0, 0);
+                    return Ops<T>::mul(in[(long long)b * a.ncols], __ldg(&twN[b * o]));
+                },
+                [](int, C v) { return v; });
             auto store = [&](int k2, C v) {
                 const int kp = out_slot(o + a.fa * k2, a.out_len, a.fN);
                 if (kp < 0 || !on) return;

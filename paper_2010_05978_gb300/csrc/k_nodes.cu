@@ -268,7 +268,7 @@ __global__ void k_petal_tables(FamilyDev f) {
 // support start and fraction, bounds, record and tile keys.
 __device__ __forceinline__ void finish_df(dflt v1, dflt v2, float cre, float cim,
                                           const ChirpParams& cp, NodeRec<float>* out,
-                                          unsigned* status, int key[4]) {
+                                          unsigned* status, int2& cell) {
     NodeRec<float> r;
     r.cre = cre;
     r.cim = cim;
@@ -295,13 +295,13 @@ __device__ __forceinline__ void finish_df(dflt v1, dflt v2, float cre, float cim
         s2 = min(max(s2, 0), cp.nf2 - cp.w);
     }
     r.s1 = s1;
-    r.s2 = s2;
+    r.s2 = s2 + cp.row_base;
     *out = r;
-    node_tiles(s1, s2, cp, key);
+    cell = make_int2(s1, s2);
 }
 
 __device__ __forceinline__ void node_df(const FamilyDev& f, const ChirpParams& cp, long long j,
-                                        NodeRec<float>* rec, unsigned* status, int key[4],
+                                        NodeRec<float>* rec, unsigned* status, int2& cell,
                                         const ScreenDev& scr) {
     // j < 2^30 (plan limit): 32-bit division
     const unsigned i = (unsigned)j / (unsigned)f.m;
@@ -326,7 +326,7 @@ __device__ __forceinline__ void node_df(const FamilyDev& f, const ChirpParams& c
         const float y = (float)f.cy + al.hi * (float)f.by[i];
         apply_screen<float>(scr, cp.screen_k, x, y, cre, cim);
     }
-    finish_df(v1, v2, cre, cim, cp, rec + f.offset + j, status, key);
+    finish_df(v1, v2, cre, cim, cp, rec + f.offset + j, status, cell);
 }
 
 // Starshade petals in the double-float form: node (k, i, l) is table entry
@@ -334,7 +334,7 @@ __device__ __forceinline__ void node_df(const FamilyDev& f, const ChirpParams& c
 // per-petal slopes (Sec. 4.2 nodes; no FP64 per node).
 __device__ __forceinline__ void node_petal_df(const FamilyDev& f, const ChirpParams& cp,
                                               long long j, NodeRec<float>* rec, unsigned* status,
-                                              int key[4], const ScreenDev& scr) {
+                                              int2& cell, const ScreenDev& scr) {
     const unsigned k = (unsigned)j / (unsigned)f.n_bdry;   // j < 2^30
     const unsigned q = (unsigned)j - k * (unsigned)f.n_bdry;
     const float4 t0 = reinterpret_cast<const float4*>(f.ptab)[2 * q];
@@ -361,7 +361,7 @@ __device__ __forceinline__ void node_petal_df(const FamilyDev& f, const ChirpPar
         }
         apply_screen<float>(scr, cp.screen_k, x, y, cre, cim);
     }
-    finish_df(v1, v2, cre, cim, cp, rec + f.offset + j, status, key);
+    finish_df(v1, v2, cre, cim, cp, rec + f.offset + j, status, cell);
 }
 
 // Double-float table of a triangle family (FP32 fast mode), from its FP64
@@ -403,7 +403,7 @@ __global__ void k_petal_df_tables(FamilyDev f, ChirpParams cp) {
 // (Sec. 4.3 with eqs. aqnod, aqwei), then the chirp phase and the grid
 // coordinate from the family's double-float constants.
 __device__ __forceinline__ void node_tri_df(const FamilyDev& f, const ChirpParams& cp, long long j,
-                                            NodeRec<float>* rec, unsigned* status, int key[4],
+                                            NodeRec<float>* rec, unsigned* status, int2& cell,
                                             const ScreenDev& scr) {
     const unsigned pp = (unsigned)(f.p * f.p);                     // j < 2^30
     const unsigned t = (unsigned)j / pp, q = (unsigned)j - t * pp;
@@ -429,13 +429,13 @@ __device__ __forceinline__ void node_tri_df(const FamilyDev& f, const ChirpParam
     if (scr.n1) apply_screen<float>(scr, cp.screen_k, x.hi, y.hi, cre, cim);
     const dflt v1 = df_add(df_mul(x, dflt{f.tk[6], f.tk[7]}), dflt{f.G0x[0], f.G0x[1]});
     const dflt v2 = df_add(df_mul(y, dflt{f.tk[8], f.tk[9]}), dflt{f.G0y[0], f.G0y[1]});
-    finish_df(v1, v2, cre, cim, cp, rec + f.offset + j, status, key);
+    finish_df(v1, v2, cre, cim, cp, rec + f.offset + j, status, cell);
 }
 
 template <typename T>
 __device__ __forceinline__ void node_generic(const FamilyDev& f, const ChirpParams& cp, long long j,
                                              NodeRec<T>* rec, double* dx, double* dy, double* dw,
-                                             unsigned* status, int key[4], const ScreenDev& scr) {
+                                             unsigned* status, int2& cell, const ScreenDev& scr) {
     double x, y, w;
     if (f.kind == FRESNEL_FAMILY_NODES) {
         x = f.params[j];
@@ -530,9 +530,9 @@ __device__ __forceinline__ void node_generic(const FamilyDev& f, const ChirpPara
         s2 = min(max(s2, 0), cp.nf2 - cp.w);
     }
     r.s1 = s1;
-    r.s2 = s2;
+    r.s2 = s2 + cp.row_base;
     rec[g] = r;
-    node_tiles(s1, s2, cp, key);
+    cell = make_int2(s1, s2);
 }
 
 // Block -> family (binary search over the block starts), then the family
@@ -581,33 +581,103 @@ __device__ __forceinline__ void load_family(const FamTable& ft, FamSmem& sm) {
 // FP32 fast mode runs the dilation families in the double-float spoke form
 // (no FP64 per node); FP64 per node otherwise.  One launch covers every
 // family of every problem of the plan.
-template <typename T>
+// STRIPS: counts and ranks under the strip keys of `ss`; else counts of every
+// tile that the support touches.
+template <typename T, bool STRIPS>
 __global__ void __launch_bounds__(kNodeThreads)
-k_nodes(FamTable ft, NodeRec<T>* rec, int* counts, double* dx, double* dy, double* dw,
-        unsigned* status) {
+k_nodes(FamTable ft, NodeRec<T>* rec, int* counts, StripSort ss, double* dx, double* dy,
+        double* dw, unsigned* status) {
     __shared__ __align__(16) FamSmem sm;
     load_family(ft, sm);
     const FamilyDev& f = sm.f;
     const long long j = (long long)(blockIdx.x - sm.b0) * blockDim.x + threadIdx.x;
-    int key[4] = {-1, -1, -1, -1};
+    int2 cell = make_int2(0, 0);
     if (j < f.n_nodes) {
         if constexpr (sizeof(T) == 4) {
             if (f.spoke && !dx)
-                node_df(f, sm.cp, j, reinterpret_cast<NodeRec<float>*>(rec), status, key, ft.scr);
+                node_df(f, sm.cp, j, reinterpret_cast<NodeRec<float>*>(rec), status, cell, ft.scr);
             else if (f.ptab && !dx)
-                node_petal_df(f, sm.cp, j, reinterpret_cast<NodeRec<float>*>(rec), status, key,
+                node_petal_df(f, sm.cp, j, reinterpret_cast<NodeRec<float>*>(rec), status, cell,
                               ft.scr);
             else if (f.tdf && !dx)
-                node_tri_df(f, sm.cp, j, reinterpret_cast<NodeRec<float>*>(rec), status, key,
+                node_tri_df(f, sm.cp, j, reinterpret_cast<NodeRec<float>*>(rec), status, cell,
                             ft.scr);
             else
-                node_generic<T>(f, sm.cp, j, rec, dx, dy, dw, status, key, ft.scr);
+                node_generic<T>(f, sm.cp, j, rec, dx, dy, dw, status, cell, ft.scr);
         } else {
-            node_generic<T>(f, sm.cp, j, rec, dx, dy, dw, status, key, ft.scr);
+            node_generic<T>(f, sm.cp, j, rec, dx, dy, dw, status, cell, ft.scr);
         }
     }
+    if constexpr (STRIPS) {
+        int key = -1;
+        if (j < f.n_nodes) {
+            const int lt = ss.live[sm.cp.tile_base + (cell.y / kTile) * sm.cp.ntx + cell.x / kTile];
+            if (lt >= 0) key = strip_key(lt, cell.x, cell.y);
+            else atomicOr(status, kStatusOverflow);   // a tile the plan's own pass did not meet
+        }
+        const int r = agg_reserve(key, ss.counts);
+        if (j < f.n_nodes) ss.rank[f.offset + j] = r;
+    } else {
+        int key[4] = {-1, -1, -1, -1};
+        if (j < f.n_nodes) node_tiles(cell.x, cell.y, sm.cp, key);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) agg_count(key[k], counts);
+        for (int k = 0; k < 4; ++k) agg_count(key[k], counts);
+    }
+}
+
+// Key starts of a strip-sorted plan: a block scans 1024 consecutive keys'
+// counts (4 per thread) and reserves their records' places with one atomic
+// add, so blocks need no order; clears the counts.
+__global__ void __launch_bounds__(256) k_strip_starts(StripSort ss) {
+    __shared__ int s_tot[8];
+    __shared__ int s_base;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int k0 = blockIdx.x * 1024 + 4 * t;   // nkeys is a multiple of 128
+    int4 c = make_int4(0, 0, 0, 0);
+    if (k0 < ss.nkeys) {
+        c = *reinterpret_cast<const int4*>(ss.counts + k0);
+        *reinterpret_cast<int4*>(ss.counts + k0) = make_int4(0, 0, 0, 0);
+    }
+    const int sum = c.x + c.y + c.z + c.w;
+    int inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) s_tot[warp] = inc;
+    __syncthreads();
+    int before = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        const int v = s_tot[w];
+        before += w < warp ? v : 0;
+        total += v;
+    }
+    if (t == 0) s_base = atomicAdd(ss.cursor, total);
+    __syncthreads();
+    if (k0 < ss.nkeys) {
+        const int p = s_base + before + inc - sum;
+        *reinterpret_cast<int4*>(ss.start + k0) = make_int4(p, p + c.x, p + c.x + c.y,
+                                                            p + c.x + c.y + c.z);
+    }
+}
+
+// Scatter of a strip-sorted plan: record j goes to its key's start plus its
+// rank.  The record's s2 counts rows over the stacked problems, so its tile
+// needs no problem.
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_scatter_strips(long long n, const NodeRec<T>* __restrict__ rec, StripSort ss,
+                 NodeRec<T>* __restrict__ sorted, unsigned* __restrict__ status) {
+    const long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (j == 0) *ss.cursor = 0;   // the starts are done: ready for the next evaluation
+    if (j >= n) return;
+    const NodeRec<T> r = rec[j];
+    const int lt = ss.live[(r.s2 / kTile) * ss.ntx + r.s1 / kTile];
+    const long long pos = lt >= 0 ? (long long)ss.start[strip_key(lt, r.s1, r.s2)] + ss.rank[j] : -1;
+    if (pos >= 0 && pos < n) sorted[pos] = r;
+    else atomicOr(status, kStatusOverflow);
 }
 
 // Scatter of a plan's records (families as in k_nodes) to every tile their
@@ -1056,12 +1126,38 @@ template <typename T>
 void launch_nodes(const FamTable& ft, int nblocks, NodeRec<T>* rec, int* counts, double* dx,
                   double* dy, double* dw, unsigned* status, cudaStream_t st) {
     if (nblocks <= 0) return;
-    k_nodes<T><<<nblocks, kNodeThreads, 0, st>>>(ft, rec, counts, dx, dy, dw, status);
+    k_nodes<T, false><<<nblocks, kNodeThreads, 0, st>>>(ft, rec, counts, StripSort{}, dx, dy, dw,
+                                                        status);
 }
 template void launch_nodes<float>(const FamTable&, int, NodeRec<float>*, int*, double*, double*,
                                   double*, unsigned*, cudaStream_t);
 template void launch_nodes<double>(const FamTable&, int, NodeRec<double>*, int*, double*,
                                    double*, double*, unsigned*, cudaStream_t);
+
+template <typename T>
+void launch_nodes_strips(const FamTable& ft, int nblocks, NodeRec<T>* rec, const StripSort& ss,
+                         double* dx, double* dy, double* dw, unsigned* status, cudaStream_t st) {
+    if (nblocks <= 0) return;
+    k_nodes<T, true><<<nblocks, kNodeThreads, 0, st>>>(ft, rec, nullptr, ss, dx, dy, dw, status);
+}
+template void launch_nodes_strips<float>(const FamTable&, int, NodeRec<float>*, const StripSort&,
+                                         double*, double*, double*, unsigned*, cudaStream_t);
+template void launch_nodes_strips<double>(const FamTable&, int, NodeRec<double>*, const StripSort&,
+                                          double*, double*, double*, unsigned*, cudaStream_t);
+
+void launch_strip_starts(const StripSort& ss, cudaStream_t st) {
+    if (ss.nkeys > 0) k_strip_starts<<<nblk(ss.nkeys, 1024), 256, 0, st>>>(ss);
+}
+
+template <typename T>
+void launch_scatter_strips(long long n, const NodeRec<T>* rec, const StripSort& ss,
+                           NodeRec<T>* sorted, unsigned* status, cudaStream_t st) {
+    if (n > 0) k_scatter_strips<T><<<nblk(n, 256), 256, 0, st>>>(n, rec, ss, sorted, status);
+}
+template void launch_scatter_strips<float>(long long, const NodeRec<float>*, const StripSort&,
+                                           NodeRec<float>*, unsigned*, cudaStream_t);
+template void launch_scatter_strips<double>(long long, const NodeRec<double>*, const StripSort&,
+                                            NodeRec<double>*, unsigned*, cudaStream_t);
 
 template <typename T>
 void launch_scatter_fams(const FamTable& ft, int nblocks, const NodeRec<T>* rec, int* cursor,
