@@ -646,8 +646,8 @@ fresnel_status eval_impl(Plan* p, const double* d_targets, long long M, void* d_
                              p->nf1, p->nf2, p->ntx, p->ntiles, p->ks, p->st);
         p->launches += p->max_split > 0 ? 3 : 2;
     } else if (p->strips) {
-        launch_spread_strips<T>((const NodeRec<T>*)p->sorted, p->N, (cx_t<T>*)p->grid, p->nf1,
-                                p->nf2, p->ks, p->st);
+        launch_spread_strips<T>((const NodeRec<T>*)p->sorted, p->N, p->ss.nkeys,
+                                (cx_t<T>*)p->grid, p->nf1, p->nf2, p->ks, p->st);
         p->launches += 1;
     } else {
         const long long spin = p->opts.max_spin == 0 ? kDefaultMaxSpin

@@ -52,7 +52,8 @@ struct StripMap {
     static constexpr int NQ = (W + 3 + 3) / 4;           // quads of a kernel row shifted by 0..3
 };
 
-template <int W>
+// DENSE: sums in two levels, a batch's and the range's (see strip_dense).
+template <int W, bool DENSE>
 __global__ void __launch_bounds__(kStripWarps * 32)
 k_spread_strips_f32(const NodeRec<float>* __restrict__ sorted, long long n, int range,
                     float2* __restrict__ grid, int nf1, int nf2, float beta, const HornerTab hz) {
@@ -71,6 +72,7 @@ k_spread_strips_f32(const NodeRec<float>* __restrict__ sorted, long long n, int 
     for (int b = W; b < M::ROWS; ++b) ck[lane][b] = make_float2(0.0f, 0.0f);
     const int cg = lane % M::COLG, rg = lane / M::COLG;
     float2 acc[M::RPL][4];
+    float2 sum[DENSE ? M::RPL : 1][4];   // DENSE: the earlier batches'
     int slot[M::RPL];                // this lane's rows relative to the open row
     const float2* ckp[M::RPL];       // their staged values (of record 0)
     const float4* kxp = reinterpret_cast<const float4*>(&kx[0][4 * cg]);
@@ -83,7 +85,10 @@ k_spread_strips_f32(const NodeRec<float>* __restrict__ sorted, long long n, int 
         slot[k] = 0;
         ckp[k] = &ck[0][0];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[k][i] = make_float2(0.0f, 0.0f);
+        for (int i = 0; i < 4; ++i) {
+            acc[k][i] = make_float2(0.0f, 0.0f);
+            if constexpr (DENSE) sum[k][i] = make_float2(0.0f, 0.0f);
+        }
     }
     // adds the rows less than d below the open one to the grid (a row's zero
     // cells too: they stay inside the grid, and testing costs more)
@@ -94,6 +99,14 @@ k_spread_strips_f32(const NodeRec<float>* __restrict__ sorted, long long n, int 
                 int y = cur_b + slot[k];
                 if (y >= yend) y -= nf2;
                 float2* dst = colp + (long long)y * nf1;
+                if constexpr (DENSE) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        acc[k][i].x += sum[k][i].x;
+                        acc[k][i].y += sum[k][i].y;
+                        sum[k][i] = make_float2(0.0f, 0.0f);
+                    }
+                }
                 asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst),
                              "f"(acc[k][0].x), "f"(acc[k][0].y), "f"(acc[k][1].x),
                              "f"(acc[k][1].y)
@@ -200,6 +213,16 @@ k_spread_strips_f32(const NodeRec<float>* __restrict__ sorted, long long n, int 
                     acc[k][3].y = fmaf(c.y, kv.w, acc[k][3].y);
                 }
             }
+        }
+        if constexpr (DENSE) {
+#pragma unroll
+            for (int k = 0; k < M::RPL; ++k)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    sum[k][i].x += acc[k][i].x;
+                    sum[k][i].y += acc[k][i].y;
+                    acc[k][i] = make_float2(0.0f, 0.0f);
+                }
         }
         __syncwarp();   // the next batch overwrites the staged values
     }
@@ -314,24 +337,40 @@ k_spread_strips_f64(const NodeRec<double>* __restrict__ sorted, long long n, int
     if (cur_a >= 0) flush(W);
 }
 
-// Records per warp: enough warps for every SM's resident set (152 x 32), at
-// least one batch and at most four: 128 consecutive additions to a cell, as
-// many as the tile kernel's warps make, so that long runs on one cell round
-// no worse (the sweep: 31 us at 224 records, 33 at 128).
-inline int strip_range(long long n) {
-    long long r = (n / (152 * 32) + 31) / 32 * 32;
+// Where the keys hold many records each (a starshade on a few cells: 35; the
+// star at F = 100: 6) every warp adds to the same cells of the grid, and each
+// addition there rounds the whole sum: longer ranges, summed in two levels so
+// that they round no worse themselves.  With one level, repeats of the sweep's
+// eight-wavelength design differed by 2.7e-6 (32 records per warp), 1.3e-6
+// (128) and 1.2e-6 (256), against the tile kernel's 0.9e-6.
+inline bool strip_dense(long long n, long long nkeys) { return n >= 16 * nkeys; }
+
+// Records per warp.  FP32: enough warps for every SM's resident set (152 x
+// 32), at least one batch and at most four: 128 consecutive additions to a
+// cell, as many as the tile kernel's warps make; eight batches where dense.
+// FP64 records cost far more than a flush: two batches per warp balance the
+// SMs (w = 13: 703 us at 128 records, 627 at 32).
+inline int strip_range(long long n, bool dense, bool dbl) {
+    if (dbl) return 64;
+    if (dense) return 256;
+    const long long r = (n / (152 * 32) + 31) / 32 * 32;
     return (int)(r < 32 ? 32 : (r > 128 ? 128 : r));
 }
 
 template <typename T, int W>
-void launch_strips_w(const NodeRec<T>* sorted, long long n, cx_t<T>* grid, int nf1, int nf2,
-                     const KernelShape& ks, cudaStream_t st) {
-    const int range = strip_range(n);
+void launch_strips_w(const NodeRec<T>* sorted, long long n, long long nkeys, cx_t<T>* grid,
+                     int nf1, int nf2, const KernelShape& ks, cudaStream_t st) {
+    const bool dense = W <= 9 && strip_dense(n, nkeys);
+    const int range = strip_range(n, dense, sizeof(T) == 8);
     const long long warps = (n + range - 1) / range;
     const int blocks = (int)((warps + kStripWarps - 1) / kStripWarps);
     if constexpr (sizeof(T) == 4) {
-        k_spread_strips_f32<W><<<blocks, kStripWarps * 32, 0, st>>>(
-            sorted, n, range, grid, nf1, nf2, ks.betaf, ks.horner);
+        if (dense)
+            k_spread_strips_f32<W, (W <= 9)><<<blocks, kStripWarps * 32, 0, st>>>(
+                sorted, n, range, grid, nf1, nf2, ks.betaf, ks.horner);
+        else
+            k_spread_strips_f32<W, false><<<blocks, kStripWarps * 32, 0, st>>>(
+                sorted, n, range, grid, nf1, nf2, ks.betaf, ks.horner);
     } else {
         const size_t smem = sizeof(StripSmemD<W>);
         cudaFuncSetAttribute(k_spread_strips_f64<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -342,12 +381,12 @@ void launch_strips_w(const NodeRec<T>* sorted, long long n, cx_t<T>* grid, int n
 }
 
 template <typename T>
-void launch_strips_impl(const NodeRec<T>* sorted, long long n, cx_t<T>* grid, int nf1, int nf2,
-                        const KernelShape& ks, cudaStream_t st) {
+void launch_strips_impl(const NodeRec<T>* sorted, long long n, long long nkeys, cx_t<T>* grid,
+                        int nf1, int nf2, const KernelShape& ks, cudaStream_t st) {
     if (n <= 0) return;
 #define FRES_STRIP_CASE(WW)                                          \
     case WW:                                                         \
-        launch_strips_w<T, WW>(sorted, n, grid, nf1, nf2, ks, st);   \
+        launch_strips_w<T, WW>(sorted, n, nkeys, grid, nf1, nf2, ks, st); \
         break;
     switch (ks.w) {
         FRES_STRIP_CASE(2) FRES_STRIP_CASE(3) FRES_STRIP_CASE(4) FRES_STRIP_CASE(5)
