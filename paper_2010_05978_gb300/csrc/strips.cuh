@@ -343,16 +343,24 @@ k_spread_strips_f64(const NodeRec<double>* __restrict__ sorted, long long n, int
 // that they round no worse themselves.  With one level, repeats of the sweep's
 // eight-wavelength design differed by 2.7e-6 (32 records per warp), 1.3e-6
 // (128) and 1.2e-6 (256), against the tile kernel's 0.9e-6.
-inline bool strip_dense(long long n, long long nkeys) { return n >= 16 * nkeys; }
+// FP64 (one level) from 64 records per key on: 311,297 nodes, a third of them
+// on one point, 1.4e-13 from the exact sums at 64 records per warp, against the tile
+// kernel's 0.4e-13.
+inline bool strip_dense(long long n, long long nkeys, bool dbl) {
+    return n >= (dbl ? 64 : 16) * nkeys;
+}
 
 // Records per warp.  FP32: enough warps for every SM's resident set (152 x
 // 32), at least one batch and at most four: 128 consecutive additions to a
 // cell, as many as the tile kernel's warps make; eight batches where dense.
-// FP64 records cost far more than a flush: two batches per warp balance the
-// SMs (w = 13: 703 us at 128 records, 627 at 32).
+// FP64 records cost far more than a flush, so the split that balances the SMs
+// wins: two batches per warp (w = 13: 703 us at 128 records, 627 at 32), one
+// below 16 warps per SM, dense or not (81,120 nodes of five starshades, w = 10:
+// 176 us at 256).
 inline int strip_range(long long n, bool dense, bool dbl) {
-    if (dbl) return 64;
+    if (dbl && n < 152LL * 16 * 64) return 32;
     if (dense) return 256;
+    if (dbl) return 64;
     const long long r = (n / (152 * 32) + 31) / 32 * 32;
     return (int)(r < 32 ? 32 : (r > 128 ? 128 : r));
 }
@@ -360,7 +368,7 @@ inline int strip_range(long long n, bool dense, bool dbl) {
 template <typename T, int W>
 void launch_strips_w(const NodeRec<T>* sorted, long long n, long long nkeys, cx_t<T>* grid,
                      int nf1, int nf2, const KernelShape& ks, cudaStream_t st) {
-    const bool dense = W <= 9 && strip_dense(n, nkeys);
+    const bool dense = (W <= 9 || sizeof(T) == 8) && strip_dense(n, nkeys, sizeof(T) == 8);
     const int range = strip_range(n, dense, sizeof(T) == 8);
     const long long warps = (n + range - 1) / range;
     const int blocks = (int)((warps + kStripWarps - 1) / kStripWarps);
