@@ -168,9 +168,10 @@ typedef struct {
     int t3_binning;
     /* FFT lengths above this run as four-step transforms fa x fb (two launches
      * per pass through an intermediate buffer) instead of one shared-memory
-     * pass; 0 = only when one pass does not fit in shared memory (lengths
-     * above ~13,600 in FP32, ~6,800 in FP64).  Batched plans and profile
-     * gradients need single-pass lengths. */
+     * pass; 0 = when one pass does not fit in shared memory (lengths above
+     * ~13,600 in FP32, ~6,800 in FP64), and for FP32 SCATTERED plans without
+     * a memory cap also columns above 2,400, where four steps are faster.
+     * Batched plans and profile gradients need single-pass lengths. */
     int fft_split_above;
     /* 1: measure before committing to a configuration.  FP64 with automatic
      * sigma / width: plans with sigma = 5/4 and 2 are built and timed on the

@@ -50,6 +50,10 @@ constexpr int kMaxEvents = 16;
 constexpr long long kSortTargetsFrom = 32768;
 constexpr long long kBinFromGridBytes = 64LL << 20;
 
+// Column transforms longer than this take four steps in FP32 scattered plans
+// (measured: see the table at launch_fft_cols).
+constexpr int kSplitColumnsAbove = 2400;
+
 // FFT along one dimension: one shared-memory pass, or four steps fa x fb
 // (A-point transforms, twiddle, B-point transforms) for longer lengths.
 struct FftDim {
@@ -57,7 +61,8 @@ struct FftDim {
     bool big = false;
     int fa = 0, fb = 0;
     FftPlan fp{}, fpa{}, fpb{};
-    void* tw = nullptr;            // w_n table (for a four-step length, the w_N twiddles)
+    void* tw = nullptr;            // w_n table (direct column DFT; the four steps' w_N twiddles)
+    void* stw = nullptr;           // stage twiddles of fp, or of fpa and fpb
     void* twa = nullptr;
     void* twb = nullptr;
 };
@@ -115,8 +120,6 @@ struct Plan {
     void* grid = nullptr;
     void* inter = nullptr;
     void* F = nullptr;
-    void* tw1 = nullptr;
-    void* tw2 = nullptr;
     void* ax = nullptr;
     void* ay = nullptr;
     void* dec1 = nullptr;
@@ -510,7 +513,7 @@ template <typename T>
 void run_rows(Plan* p, RowPassArgs ra) {
     const FftDim& d = p->d1;
     if (!d.big) {
-        ra.twiddle = d.tw;
+        ra.twiddle = d.stw;
         launch_fft_rows<T>(d.fp, ra, p->st);
         p->launches++;
         return;
@@ -557,7 +560,7 @@ template <typename T>
 void run_cols(Plan* p, ColPassArgs ca) {
     const FftDim& d = p->d2;
     if (!d.big) {
-        ca.twiddle = d.tw;
+        ca.twiddle = d.stw;
         launch_fft_cols<T>(d.fp, ca, p->st);
         p->launches++;
         return;
@@ -683,7 +686,6 @@ fresnel_status eval_impl(Plan* p, const double* d_targets, long long M, void* d_
         ca.in_len = p->nf2;
         ca.centered_in = 0;
         ca.out_len = p->n2;
-        ca.twiddle = p->tw2;
         ca.ax = p->ax;
         ca.ay = p->ay;
         ca.occulter = p->output == FRESNEL_OCCULTER;
@@ -1071,7 +1073,6 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
     choose_kernel(p);
     const int w = p->ks.w;
     const double lz = p->lz;
-    int cmax = 0;
     p->cp.kq = kPi / lz;
     p->cp.w = w;
     if (p->tkind == FRESNEL_GRID) {
@@ -1150,12 +1151,18 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
     for (FftDim* d : {&p->d1, &p->d2}) {
         d->n = d == &p->d1 ? p->nfft1 : p->nfft2;
         const bool forced = p->opts.fft_split_above > 0 && d->n > p->opts.fft_split_above;
-        if (fft_supported(d->n, dbl, &cmax) && !forced) {
-            d->fp = make_fft_plan(d->n, dbl ? 8 : 16);
+        // FP32 scattered plans (one problem, no gradients: nothing else needs
+        // single passes) split long columns too: a single pass takes two
+        // columns per block there, 16 of a sector's 32 bytes
+        const bool split_cols = d == &p->d2 && !dbl && p->tkind == FRESNEL_SCATTERED &&
+                                p->opts.fft_split_above == 0 && p->opts.max_device_bytes == 0 &&
+                                d->n > kSplitColumnsAbove && fft_split(d->n, dbl, &d->fa, &d->fb);
+        if (fft_supported(d->n, dbl) && !forced && !split_cols) {
+            d->fp = make_fft_plan(d->n, dbl);
         } else if (fft_split(d->n, dbl, &d->fa, &d->fb)) {
             d->big = true;
-            d->fpa = make_fft_plan(d->fa, dbl ? 8 : 16);
-            d->fpb = make_fft_plan(d->fb, dbl ? 8 : 16);
+            d->fpa = make_fft_plan(d->fa, dbl);
+            d->fpb = make_fft_plan(d->fb, dbl);
         } else {
             return fres_fail(FRESNEL_ERR_UNSUPPORTED, "FFT length " + std::to_string(d->n) +
                                                           " has no supported split");
@@ -1549,14 +1556,15 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
         FRES_TRY(dalloc(p, &d->tw, cs * d->n));
         launch_twiddles(d->n, d->tw, dbl, p->st);
         if (d->big) {
-            FRES_TRY(dalloc(p, &d->twa, cs * d->fa));
-            launch_twiddles(d->fa, d->twa, dbl, p->st);
-            FRES_TRY(dalloc(p, &d->twb, cs * d->fb));
-            launch_twiddles(d->fb, d->twb, dbl, p->st);
+            FRES_TRY(dalloc(p, &d->twa, cs * d->fpa.ntw));
+            launch_stage_twiddles(d->fpa, d->twa, dbl, p->st);
+            FRES_TRY(dalloc(p, &d->twb, cs * d->fpb.ntw));
+            launch_stage_twiddles(d->fpb, d->twb, dbl, p->st);
+        } else {
+            FRES_TRY(dalloc(p, &d->stw, cs * d->fp.ntw));
+            launch_stage_twiddles(d->fp, d->stw, dbl, p->st);
         }
     }
-    p->tw1 = p->d1.tw;
-    p->tw2 = p->d2.tw;
     if (p->d1.big || p->d2.big) {   // four-step intermediate, shared by both passes
         const size_t rows = p->d1.big ? (size_t)p->nf2 * p->d1.n : 0;
         const size_t ncol = p->tkind == FRESNEL_GRID ? (size_t)p->n1 : (size_t)p->nfft1;
@@ -1662,7 +1670,7 @@ fresnel_status adjoint_grid(Plan* p, const void* d_gamma) {
     ra.in_len = p->n1;
     ra.centered_in = 1;
     ra.out_len = p->nf1;
-    ra.twiddle = p->tw1;
+    ra.twiddle = p->d1.stw;
     launch_fft_rows<T>(p->fp1, ra, p->st);
     ColPassArgs ca{};
     ca.in = p->adj_rows;
@@ -1671,7 +1679,7 @@ fresnel_status adjoint_grid(Plan* p, const void* d_gamma) {
     ca.in_len = p->n2;
     ca.centered_in = 1;
     ca.out_len = p->nf2;
-    ca.twiddle = p->tw2;
+    ca.twiddle = p->d2.stw;
     ca.out_is_final = 0;
     ca.batch = p->B;
     ca.in_bstride = (long long)p->n2 * p->nf1;

@@ -13,7 +13,7 @@ namespace fres {
 
 constexpr int kMaxW = 16;          // widest spreading kernel supported
 constexpr int kTile = 32;          // spreading tile edge (grid points)
-constexpr int kMaxRadixStages = 32;
+constexpr int kMaxRadixStages = 12;
 constexpr int kMaxCheb = 64;       // Chebyshev terms kept for psihat (type 3)
 constexpr double kTwoPi = 6.283185307179586476925286766559;
 constexpr double kPi = 3.141592653589793238462643383280;
@@ -75,11 +75,16 @@ __host__ __device__ __forceinline__ int split_code(int split_index, bool first) 
     return ((split_index + 1) << 1) | (first ? 1 : 0);
 }
 
-// Radix plan of one FFT length.
+// Radix plan of one FFT length (at least two stages).
 struct FftPlan {
     int n;
     int nstages;
+    int threads;                   // threads per line (each keeps up to 16 values, FP64 10)
+    int ntw;                       // entries of the stage twiddle table
     int radix[kMaxRadixStages];
+    int nb[kMaxRadixStages];       // butterflies of the stage: n / radix
+    // stage s > 0: w_{p radix}^{q k} at toff + (q - 1) p + k (0 < q < radix, k < p)
+    int toff[kMaxRadixStages];
     // stage s: p = product of the earlier radices and ceil(2^32 / p), so that
     // i / p = umulhi(i, pmagic) exactly for i * p < 2^32 (p = 1: magic 0)
     int p[kMaxRadixStages];
@@ -351,6 +356,8 @@ template <typename T>
 void launch_scatter(long long n, const ChirpParams& cp, const NodeRec<T>* rec, int* cursor,
                     NodeRec<T>* sorted, long long cap, unsigned* status, cudaStream_t st);
 void launch_twiddles(int n, void* table, int is_double, cudaStream_t st);
+// the stage twiddles of fp (fp.ntw entries)
+void launch_stage_twiddles(const FftPlan& fp, void* table, int is_double, cudaStream_t st);
 // t1 output tables Ax[k1] = chirp(xi)/(i lz)/psihat(k1), Ay[k2] = chirp(eta)/psihat(k2),
 // each times exp(2 pi i k shift / nf) for a grid spread shifted by shift cells
 void launch_t1_tables(int n, int nf, double h, double x0, double lz, int w, double beta,
@@ -423,7 +430,7 @@ struct RowPassArgs {
     const void* deconv_col;   // per-element factor along the row (centered_in), or NULL
     const void* deconv_row;   // per-row scalar factor (centered_in), or NULL
     int out_len;         // kept outputs: modes k in [-out_len/2, out_len - out_len/2), stored at k + out_len/2 (out_len == n: fftshifted)
-    const void* twiddle;
+    const void* twiddle;   // stage twiddles
     // rows of dead tile rows (live[(row / batch_rows) * nty + (row % batch_rows) / 32] == 0)
     // are skipped: neither read nor written.  NULL: every row is live.
     const int* live;
@@ -497,10 +504,10 @@ void launch_col_dft_tc(const ColPassArgs& a, int n, unsigned* status, cudaStream
 // rows twiddled by w_n^{b j} (n a multiple of 32, at most 32768)
 bool col_pfft_supported(int n, int live_rows);
 void launch_col_pfft_d(const ColPassArgs& a, int n, unsigned* status, cudaStream_t st);
-bool fft_supported(int n, int is_double, int* max_cols);
+bool fft_supported(int n, int is_double);
 // Split of a length beyond one pass into fa * fb (both single-pass), or false.
 bool fft_split(int n, int is_double, int* fa, int* fb);
-FftPlan make_fft_plan(int n, int max_radix);
+FftPlan make_fft_plan(int n, int is_double);   // nstages < 0: no plan
 
 // k_interp.cu
 struct InterpParams {

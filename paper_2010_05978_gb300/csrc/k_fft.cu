@@ -1,7 +1,7 @@
-// Hand-written 2D FFT for the NUFFT fine grid: batched 1D mixed-radix
-// (4, 2, 3, 5) Stockham transforms held in shared memory, one pass along rows
-// (contiguous) and one along columns (a CTA takes C adjacent columns so global
-// accesses stay coalesced).  Forward sign e^{-2 pi i k l / n}, unnormalised.
+// Hand-written 2D FFT for the NUFFT fine grid: batched 1D mixed-radix Stockham
+// transforms held in shared memory, one pass along rows (contiguous) and one
+// along columns (a CTA takes several adjacent columns so global accesses stay
+// coalesced).  Forward sign e^{-2 pi i k l / n}, unnormalised.
 //
 // The FFT is the middle step of the type-1 and type-3 NUFFTs used by the
 // paper's fast algorithm (arXiv:2010.05978, Secs. 3.2-3.3; "under the hood the
@@ -13,20 +13,39 @@
 //
 // Each Stockham stage with radix r and p = product of earlier radices maps
 // butterfly i (k = i mod p) from inputs x[i + q n/r] (twiddled by
-// w_n^{q k n/(p r)}) to outputs y[(i - k) r + k + t p]; stages ping-pong
-// between two shared-memory buffers with one barrier each.  The first stage
-// reads its inputs straight from global memory and the last writes its
-// outputs straight to global memory (through the pruning and the epilogue),
-// so a transform makes no separate staging passes.
+// w_{p r}^{q k}) to outputs y[(i - k) r + k + t p].  A thread keeps up
+// to 16 values (FP64: 8): several butterflies of a small radix, read into registers
+// before a barrier and written back in place after it, so one buffer per line
+// is enough and the threads (64 registers) and lines resident at once cover
+// the passes' grids in one wave.  These passes are short and bound by latency:
+// fewer stages (radices up to 16 with the composite 15, 12, 10 and 9, which
+// need no inner twiddles but 9's and 16's) and twiddles read consecutively from a table
+// per stage matter more than operations, and so does the code a block
+// runs once: in the single passes one body per radix serves every stage, with
+// the pruning, factors and epilogue in the short loops that fill and empty
+// the lines (fused into the first and last stages they made 33 KB of
+// straight-line code, whose fetching took up to half of a pass: 29 against 19
+// us cold for the star's 928 rows of 2048).  The four-step passes are short
+// transforms over gigabytes: there the code stays fetched, and they read and
+// store in their first and last stages (17,280^2 points: 3.6 against 4.8 ms).
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace fres {
 
 namespace {
 
-constexpr int kFftThreads = 256;
-constexpr int kFftBlocksPerSm = 3;
-constexpr long long kFftSmemTarget = 76 * 1024;   // three blocks per SM
+// Radices, and the butterflies of a radix that a thread keeps: 16 values in
+// FP32; 8 in FP64 (9 and 10 for the radices 3 and 5, so that lines of up to
+// 6,834 points need no more than 1024 threads whatever their factors; 16
+// values and the larger radices save a quarter of FP64's twiddles, but leave
+// a short line too few warps: 720 points 49 against 41 us).
+constexpr int kRadicesF[] = {16, 15, 12, 10, 9, 8, 5, 4, 3, 2};
+constexpr int kRadicesD[] = {8, 6, 5, 4, 3, 2};
+__host__ __device__ constexpr int butterflies(int r, bool dbl) {
+    return dbl ? (r == 3 ? 3 : (r == 5 ? 2 : 8 / r > 0 ? 8 / r : 1)) : 16 / r;
+}
 
 template <typename T> struct Ops {
     using C = cx_t<T>;
@@ -156,108 +175,230 @@ template <typename T> struct Dft<T, 16> {
     }
 };
 
+// Coprime composites N = N1 N2 by the prime-factor map: input (N2 a + N1 b)
+// mod N, output k at (k mod N1, k mod N2), no twiddles.
+template <typename T, int N1, int N2> struct DftPfa {
+    using C = cx_t<T>;
+    static __device__ __forceinline__ void run(const C* u, C* y) {
+        constexpr int N = N1 * N2;
+        C A[N2][N1];
+#pragma unroll
+        for (int b = 0; b < N2; ++b) {
+            C v[N1];
+#pragma unroll
+            for (int a = 0; a < N1; ++a) v[a] = u[(N2 * a + N1 * b) % N];
+            Dft<T, N1>::run(v, A[b]);
+        }
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) {
+            C v[N2], d[N2];
+#pragma unroll
+            for (int b = 0; b < N2; ++b) v[b] = A[b][k1];
+            Dft<T, N2>::run(v, d);
+#pragma unroll
+            for (int k = 0; k < N; ++k)
+                if (k % N1 == k1) y[k] = d[k % N2];
+        }
+    }
+};
+template <typename T> struct Dft<T, 6> : DftPfa<T, 2, 3> {};
+template <typename T> struct Dft<T, 10> : DftPfa<T, 2, 5> {};
+template <typename T> struct Dft<T, 12> : DftPfa<T, 4, 3> {};
+template <typename T> struct Dft<T, 15> : DftPfa<T, 3, 5> {};
+template <typename T> struct Dft<T, 9> {
+    using C = cx_t<T>;
+    static __device__ __forceinline__ void run(const C* u, C* y) {
+        using O = Ops<T>;
+        // cos / sin of 2 pi j / 9, j = 0..4 (j = n2 k1 takes 1, 2, 4)
+        const T cs[5] = {(T)1, (T)0.76604444311897803520239265055542,
+                         (T)0.17364817766693034885171662676931, (T)-0.5,
+                         (T)-0.93969262078590838405410927732473};
+        const T sn[5] = {(T)0, (T)0.64278760968653932632264340990726,
+                         (T)0.98480775301220805936674302458952,
+                         (T)0.86602540378443864676372317075294,
+                         (T)0.34202014332566873304409961468226};
+        C A[3][3];
+#pragma unroll
+        for (int n2 = 0; n2 < 3; ++n2) {
+            C v[3] = {u[n2], u[3 + n2], u[6 + n2]};
+            Dft<T, 3>::run(v, A[n2]);
+#pragma unroll
+            for (int k1 = 1; k1 < 3; ++k1)
+                if (n2 > 0) A[n2][k1] = O::mul(A[n2][k1], O::mk(cs[n2 * k1], -sn[n2 * k1]));
+        }
+#pragma unroll
+        for (int k1 = 0; k1 < 3; ++k1) {
+            C v[3] = {A[0][k1], A[1][k1], A[2][k1]}, d[3];
+            Dft<T, 3>::run(v, d);
+#pragma unroll
+            for (int k2 = 0; k2 < 3; ++k2) y[k1 + 3 * k2] = d[k2];
+        }
+    }
+};
+
 // Shared-memory element index with one padding slot per 16 elements, so the
 // stride-R writes of the early Stockham stages spread over all banks.
 __host__ __device__ __forceinline__ int pad(int e) { return e + (e >> 4); }
 __host__ __device__ __forceinline__ int padded_len(int n) { return n + (n >> 4) + 1; }
 
-template <typename T> __host__ __device__ constexpr int emax() { return 8; }
+// A thread's place: its line (c: offset of the line's element 0 in S, element
+// e at c + (pad(e) << ls)) and its butterflies or elements t, t + tr, ...
+struct Place {
+    int c, t, tr, ls;
+};
 
-// The input side of a transform: load(e) reads natural input e, use(e, v)
-// turns the value read into the value transformed (a factor, and where asked
-// for the input set back to zero).  Apart, so that a butterfly's loads are
-// all in flight before a store that may alias them: with the zeroing inside
-// the load the 64-wavelength sweep's row pass took 35 us instead of 21.
+// The input side of a fused transform: load(e) reads natural input e, use(e,
+// v) turns the value read into the value transformed.  Apart, so that a
+// butterfly's loads are all in flight before a store that may alias them.
 template <class L, class U>
 struct Input {
     L l;
     U u;
-    __device__ __forceinline__ auto operator()(int e) const { return l(e); }
+    __device__ __forceinline__ auto load(int e) const { return l(e); }
     template <class C> __device__ __forceinline__ C use(int e, C v) const { return u(e, v); }
 };
 template <class L, class U> __device__ __forceinline__ Input<L, U> make_input(L l, U u) { return {l, u}; }
+struct NoIo {
+    template <class C> __device__ __forceinline__ void operator()(int, C) const {}
+};
 
-// A stage whose inputs come from global memory (FIRST: load(e) for natural
-// input index e, always p = 1) and/or whose outputs go straight to global
-// memory (LAST: store(k, value) for natural output index k); otherwise as
-// stage().  Fusing the first and last stages with the loads and stores saves
-// two shared-memory round trips and two barriers per transform.
-template <typename T, int R, int NCOL, bool FIRST, bool LAST, class Load, class Store>
-__device__ __forceinline__ void stage_io(const cx_t<T>* __restrict__ src, cx_t<T>* __restrict__ dst,
-                                         int n, int p, unsigned pmagic,
-                                         const cx_t<T>* __restrict__ tw, Load& load, Store& store) {
+// One stage, in place: every butterfly of the line is read before any is
+// written.  kStage: from S to S; kFirst: from `in` (p = 1) to S; kLast: from S
+// to `out` (output i + t p of butterfly i).
+enum { kStage = 0, kFirst = 1, kLast = 2 };
+template <typename T, int R, int WHERE, class In, class Out>
+__device__ __forceinline__ void stage(cx_t<T>* __restrict__ S, const Place pl, int nb, int p,
+                                      unsigned pmagic, const cx_t<T>* __restrict__ tw, In& in,
+                                      Out& out) {
     using O = Ops<T>;
     using C = cx_t<T>;
-    const int nb = n / R;
-    const int items = nb * NCOL;
-    const int twstep = n / (p * R);
-    for (int w = threadIdx.x; w < items; w += blockDim.x) {
-        const int c = w & (NCOL - 1), i = w / NCOL;
-        const int k = (FIRST || p == 1) ? 0 : i - (int)__umulhi((unsigned)i, pmagic) * p;
-        const int kt = k * twstep;
-        C u[R], y[R];
+    constexpr int K = butterflies(R, sizeof(T) == 8);
+    C u[K][R];
 #pragma unroll
-        for (int q = 0; q < R; ++q) {
-            if constexpr (FIRST) {
-                u[q] = load(i + q * nb);   // all R loads in flight before the first use
-            } else {
-                u[q] = src[pad(i + q * nb) * NCOL + c];
-                if (q > 0 && k > 0) u[q] = O::mul(u[q], __ldg(&tw[q * kt]));
+    for (int kk = 0; kk < K; ++kk) {
+        const int i = pl.t + kk * pl.tr;
+        if (i < nb) {
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                if constexpr (WHERE == kFirst) u[kk][q] = in.load(i + q * nb);
+                else u[kk][q] = S[pl.c + (pad(i + q * nb) << pl.ls)];
+            }
+        } else {   // defined on every path: else a value carried round the stage loop, and spilled
+#pragma unroll
+            for (int q = 0; q < R; ++q) u[kk][q] = O::mk(0, 0);
+        }
+    }
+    if constexpr (WHERE != kFirst) __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < K; ++kk) {
+        const int i = pl.t + kk * pl.tr;
+        if (i < nb) {
+            int k = 0;
+            if constexpr (WHERE == kFirst) {
+#pragma unroll
+                for (int q = 0; q < R; ++q) u[kk][q] = in.use(i + q * nb, u[kk][q]);
+            } else if (WHERE == kLast || p > 1) {
+                k = WHERE == kLast ? i : i - (int)__umulhi((unsigned)i, pmagic) * p;
+#pragma unroll
+                for (int q = 1; q < R; ++q) {
+                    // 32-bit offsets from a uniform base keep the addresses out of register pairs
+                    const unsigned off = (unsigned)((q - 1) * p + k) * (unsigned)sizeof(C);
+                    u[kk][q] = O::mul(u[kk][q], __ldg(reinterpret_cast<const C*>(
+                                                    reinterpret_cast<const char*>(tw) + off)));
+                }
+            }
+            C y[R];
+            Dft<T, R>::run(u[kk], y);
+            const int j = (i - k) * R + k;
+#pragma unroll
+            for (int t = 0; t < R; ++t) {
+                if constexpr (WHERE == kLast) out(i + t * p, y[t]);
+                else S[pl.c + (pad(j + t * p) << pl.ls)] = y[t];
             }
         }
-        if constexpr (FIRST) {
-#pragma unroll
-            for (int q = 0; q < R; ++q) u[q] = load.use(i + q * nb, u[q]);
-        }
-        Dft<T, R>::run(u, y);
-        const int j = (i - k) * R + k;
-#pragma unroll
-        for (int t = 0; t < R; ++t) {
-            if constexpr (LAST) store(j + t * p, y[t]);
-            else dst[pad(j + t * p) * NCOL + c] = y[t];
-        }
     }
-    __syncthreads();
+    if constexpr (WHERE != kLast) __syncthreads();
 }
 
-template <typename T, int NCOL, bool FIRST, bool LAST, class Load, class Store>
-__device__ __forceinline__ void stage_dispatch(int r, const cx_t<T>* src, cx_t<T>* dst, int n, int p,
-                                               unsigned mg, const cx_t<T>* tw, Load& load,
-                                               Store& store) {
-    switch (r) {
-        case 16:
-            if constexpr (sizeof(T) == 4)
-                stage_io<T, 16, NCOL, FIRST, LAST>(src, dst, n, p, mg, tw, load, store);
-            break;
-        case 8: stage_io<T, 8, NCOL, FIRST, LAST>(src, dst, n, p, mg, tw, load, store); break;
-        case 4: stage_io<T, 4, NCOL, FIRST, LAST>(src, dst, n, p, mg, tw, load, store); break;
-        case 2: stage_io<T, 2, NCOL, FIRST, LAST>(src, dst, n, p, mg, tw, load, store); break;
-        case 3: stage_io<T, 3, NCOL, FIRST, LAST>(src, dst, n, p, mg, tw, load, store); break;
-        case 5: stage_io<T, 5, NCOL, FIRST, LAST>(src, dst, n, p, mg, tw, load, store); break;
+template <typename T, int WHERE, class In, class Out>
+__device__ __forceinline__ void stage_dispatch(int s, const FftPlan& fp, cx_t<T>* S, const Place pl,
+                                               const cx_t<T>* tw, In& in, Out& out) {
+    const int nb = fp.nb[s], p = fp.p[s];
+    const unsigned mg = fp.pmagic[s];
+    const cx_t<T>* t = tw + fp.toff[s];
+#define FRES_RADIX(RR)                                                     \
+    case RR: stage<T, RR, WHERE>(S, pl, nb, p, mg, t, in, out); break;
+    if constexpr (sizeof(T) == 4) {
+        switch (fp.radix[s]) {
+            FRES_RADIX(16) FRES_RADIX(15) FRES_RADIX(12) FRES_RADIX(10) FRES_RADIX(9)
+            FRES_RADIX(8) FRES_RADIX(5) FRES_RADIX(4) FRES_RADIX(3) FRES_RADIX(2)
+        }
+    } else {
+        switch (fp.radix[s]) {
+            FRES_RADIX(8) FRES_RADIX(6) FRES_RADIX(5) FRES_RADIX(4) FRES_RADIX(3) FRES_RADIX(2)
+        }
+    }
+#undef FRES_RADIX
+}
+
+// The transform of the lines in S.  Every thread of the block must call it
+// (it holds barriers).  A block transforms its lines once: in a loop over
+// lines the compiler keeps the stages' invariant twiddles in registers, and
+// spills.
+template <typename T>
+__device__ __forceinline__ void fft_line(cx_t<T>* S, const FftPlan& fp, const Place pl,
+                                         const cx_t<T>* tw) {
+    NoIo none;
+    for (int s = 0; s < fp.nstages; ++s) stage_dispatch<T, kStage>(s, fp, S, pl, tw, none, none);
+}
+// The same from `in` to `out`, the first stage at place pf.
+template <typename T, class In, class Out>
+__device__ __forceinline__ void fft_fused(cx_t<T>* S, const FftPlan& fp, const Place pf,
+                                          const Place pl, const cx_t<T>* tw, In& in, Out& out) {
+    stage_dispatch<T, kFirst>(0, fp, S, pf, tw, in, out);
+    for (int s = 1; s < fp.nstages - 1; ++s) stage_dispatch<T, kStage>(s, fp, S, pl, tw, in, out);
+    stage_dispatch<T, kLast>(fp.nstages - 1, fp, S, pl, tw, in, out);
+}
+
+// Natural index of input i of len (centred: modes i - len/2), and of kept
+// output kp (centred order over len).
+__device__ __forceinline__ int in_natural(int i, int len, int n, int centered) {
+    if (!centered) return i;
+    return i < len / 2 ? n - len / 2 + i : i - len / 2;
+}
+__device__ __forceinline__ int out_natural(int kp, int len, int n) {
+    return kp < len / 2 ? n - len / 2 + kp : kp - len / 2;
+}
+
+// items t, t + tr, ... below count, kBatch at a time: read all, then use all,
+// so that a batch's loads are in flight together.
+template <typename C, class Read, class Use>
+__device__ __forceinline__ void batched(const Place pl, int count, Read read, Use use) {
+    constexpr int kBatch = sizeof(C) == 8 ? 8 : 4;
+#pragma unroll 1
+    for (int i0 = pl.t; i0 < count; i0 += kBatch * pl.tr) {
+        C v[kBatch];
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            const int i = i0 + b * pl.tr;
+            if (i < count) v[b] = read(i);
+        }
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            const int i = i0 + b * pl.tr;
+            if (i < count) use(i, v[b]);
+        }
     }
 }
 
-// The whole transform with the first stage reading load(e) and the last
-// writing store(k, v) (natural indices); A and B are the shared ping-pong
-// buffers.  Every thread of the block must call it (it holds barriers).
-template <typename T, int NCOL, class Load, class Store>
-__device__ void fft_fused(cx_t<T>* A, cx_t<T>* B, const FftPlan& fp, const cx_t<T>* tw, Load& load,
-                          Store& store) {
-    const int S = fp.nstages;
-    if (S == 1) {
-        stage_dispatch<T, NCOL, true, true>(fp.radix[0], A, B, fp.n, 1, 0u, tw, load, store);
-        return;
-    }
-    stage_dispatch<T, NCOL, true, false>(fp.radix[0], A, A, fp.n, 1, 0u, tw, load, store);
-    for (int s = 1; s < S - 1; ++s) {
-        stage_dispatch<T, NCOL, false, false>(fp.radix[s], A, B, fp.n, fp.p[s], fp.pmagic[s], tw,
-                                              load, store);
-        cx_t<T>* t = A;
-        A = B;
-        B = t;
-    }
-    stage_dispatch<T, NCOL, false, true>(fp.radix[S - 1], A, B, fp.n, fp.p[S - 1],
-                                         fp.pmagic[S - 1], tw, load, store);
+// The line's elements that no input fills: [in natural order] after the
+// inputs, or between the centred inputs' two halves.
+template <typename C>
+__device__ __forceinline__ void zero_rest(C* S, const Place pl, int len, int n, int centered) {
+    C z;
+    z.x = z.y = 0;
+    const int lo = centered ? len - len / 2 : len, hi = centered ? n - len / 2 : n;
+    for (int e = lo + pl.t; e < hi; e += pl.tr) S[pl.c + (pad(e) << pl.ls)] = z;
 }
 
 // Natural input index e of a length-n transform whose len inputs hold modes
@@ -276,287 +417,297 @@ __device__ __forceinline__ int out_slot(int k, int len, int n) {
     return -1;
 }
 
-
-
+// Rows: a block takes `lines` rows, tr threads each.
 template <typename T>
-__global__ void __launch_bounds__(kFftThreads, kFftBlocksPerSm)
-k_fft_rows(FftPlan fp, RowPassArgs a) {
+__global__ void __launch_bounds__(1024, 1)
+k_fft_rows(FftPlan fp, RowPassArgs a, int lines, int tr) {
     using C = cx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* S = (C*)smem_raw;
-    C* S2 = S + padded_len(fp.n);
     const int n = fp.n;
     const C* tw = (const C*)a.twiddle;
     const T* dcol = (const T*)a.deconv_col;
-    // rows of dead tile rows are zero in and out of the transform: skipped,
-    // through the plan's list of live rows when it has one, else by the rows'
-    // live flags
-    auto next_live = [&](int r) {
-        if (a.live)
-            while (r < a.nrows && !a.live[(r / a.batch_rows) * a.nty + (r % a.batch_rows) / kTile])
-                r += gridDim.x;
-        return r;
-    };
-    auto transform = [&](int row) {
-        C* in = (C*)a.in + (long long)row * a.in_stride;
-        C* out = (C*)a.out + (long long)row * a.out_stride;
-        const T rowf = a.deconv_row ? ((const T*)a.deconv_row)[row] : (T)1;
-        auto load = make_input(
-            [&](int e) {
-                const int i = in_src(e, a.in_len, n, a.centered_in);
-                if (i < 0) return Ops<T>::mk(0, 0);
-                C v = in[i];
-                if (a.centered_in) {
-                    if (a.clear_in && (v.x != (T)0 || v.y != (T)0)) in[i] = Ops<T>::mk(0, 0);
-                    v = Ops<T>::scale(v, rowf * (dcol ? dcol[i] : (T)1));
-                }
-                return v;
-            },
-            [&](int e, C v) {
-                if (a.clear_in && !a.centered_in && (v.x != (T)0 || v.y != (T)0) && e < a.in_len)
-                    in[e] = Ops<T>::mk(0, 0);
-                return v;
-            });
-        auto store = [&](int k, C v) {
-            const int kp = out_slot(k, a.out_len, n);
-            if (kp >= 0) out[kp] = v;
-        };
-        fft_fused<T, 1>(S, S2, fp, tw, load, store);
-    };
+    int line = threadIdx.x / tr;
+    Place pl{line * padded_len(n), (int)threadIdx.x - line * tr, tr, 0};
+    const int total = a.row_list ? a.nlist : a.nrows;
+    int row = blockIdx.x * lines + line;
+    bool on = line < lines && row < total;
     if (a.row_list) {
-        for (int i = blockIdx.x; i < a.nlist; i += gridDim.x) transform(a.row_list[i]);
-    } else {
-        for (int row = next_live(blockIdx.x); row < a.nrows; row = next_live(row + gridDim.x))
-            transform(row);
+        row = on ? a.row_list[row] : 0;
+    } else if (a.live && on) {
+        // rows of dead tile rows are zero in and out of the transform: skipped
+        on = a.live[(row / a.batch_rows) * a.nty + (row % a.batch_rows) / kTile] != 0;
+        if (lines == 1 && !on) return;   // the same for the whole block
     }
+    if (!on) {   // no line: no elements, no butterflies
+        pl.t = n;
+        pl.c = 0;
+        row = 0;
+    }
+    C* in = (C*)a.in + (long long)row * a.in_stride;
+    C* out = (C*)a.out + (long long)row * a.out_stride;
+    const T rowf = a.deconv_row ? ((const T*)a.deconv_row)[row] : (T)1;
+    batched<C>(
+        pl, a.in_len, [&](int i) { return in[i]; },
+        [&](int i, C v) {
+            if (a.clear_in && (v.x != (T)0 || v.y != (T)0)) in[i] = Ops<T>::mk(0, 0);
+            if (a.centered_in) v = Ops<T>::scale(v, rowf * (dcol ? __ldg(&dcol[i]) : (T)1));
+            S[pl.c + pad(in_natural(i, a.in_len, n, a.centered_in))] = v;
+        });
+    zero_rest(S, pl, a.in_len, n, a.centered_in);
+    __syncthreads();
+    fft_line<T>(S, fp, pl, tw);
+    for (int kp = pl.t; kp < a.out_len; kp += tr) out[kp] = S[pl.c + pad(out_natural(kp, a.out_len, n))];
 }
 
-template <typename T, int NCOL, int MODE>
-__global__ void __launch_bounds__(kFftThreads, kFftBlocksPerSm)
-k_fft_cols(FftPlan fp, ColPassArgs a) {
+// Columns: a block takes 2^ls adjacent columns.
+template <typename T, int MODE>
+__global__ void __launch_bounds__(1024, 1)
+k_fft_cols(FftPlan fp, ColPassArgs a, int ls) {
     using C = cx_t<T>;
+    using O = Ops<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ unsigned s_live[kMaxTileRows / 32];
     C* S = (C*)smem_raw;
-    C* S2 = S + padded_len(fp.n) * NCOL;
     const int n = fp.n;
     const C* tw = (const C*)a.twiddle;
-    const int ngroups = (a.ncols + NCOL - 1) / NCOL;
-    const int nouter = MODE == kFftPlain ? max(a.batch, 1) : a.nouter;
-    const int total = ngroups * nouter;            // (outer index, column group) work items
-    const int c = threadIdx.x & (NCOL - 1);        // this thread's column in every group
-    for (int gg = blockIdx.x; gg < total; gg += gridDim.x) {
-        const int o = gg / ngroups, col = (gg - o * ngroups) * NCOL + c;
-        const bool on = col < a.ncols;
-        if constexpr (MODE == kFftPlain) {
-            const int bi = o;
-            const C* in = (const C*)a.in + (long long)bi * a.in_bstride + col;
-            C* out = (C*)a.out + (long long)bi * a.out_bstride + col;
-            if (a.live) {   // live tile rows of this transform as a bit mask
-                for (int t = threadIdx.x; t < kMaxTileRows / 32; t += blockDim.x) s_live[t] = 0u;
-                __syncthreads();
-                for (int t = threadIdx.x; t < a.nty; t += blockDim.x)
-                    if (a.live[(long long)bi * a.nty + t]) atomicOr(&s_live[t >> 5], 1u << (t & 31));
-                __syncthreads();
-            }
-            C axc = Ops<T>::mk(1, 0);
-            const C* ay = nullptr;
-            if (a.ax && on) {
-                axc = ((const C*)a.ax)[(long long)bi * a.ncols + col];
-                ay = (const C*)a.ay + (long long)bi * a.out_len;
-            }
-            auto load = make_input(
-                [&](int e) {
-                    const int i = in_src(e, a.in_len, n, a.centered_in);
-                    if (i < 0 || !on) return Ops<T>::mk(0, 0);
-                    if (a.live) {
-                        const int tr = i / kTile;
-                        if (!((s_live[tr >> 5] >> (tr & 31)) & 1u)) return Ops<T>::mk(0, 0);
-                    }
-                    return in[(long long)i * a.ncols];
-                },
-                [](int, C v) { return v; });
-            auto store = [&](int k, C v) {
-                const int kp = out_slot(k, a.out_len, n);
-                if (kp < 0 || !on) return;
-                if (ay) {
-                    v = Ops<T>::mul(Ops<T>::mul(v, axc), __ldg(&ay[kp]));
-                    if (a.occulter) v = Ops<T>::mk((T)1 - v.x, -v.y);
-                }
-                out[(long long)kp * a.ncols] = v;
-            };
-            fft_fused<T, NCOL>(S, S2, fp, tw, load, store);
-        } else if constexpr (MODE == kFftRowStep1) {
-            // grid row o viewed as fa x fb (element e = fb a + b at column b = col)
-            C* in = (C*)a.in + (long long)o * a.in_stride;
-            C* out = (C*)a.out + (long long)o * a.fN + col;
-            const T rowf = a.deconv_row ? ((const T*)a.deconv_row)[o] : (T)1;
-            const T* dcol = (const T*)a.deconv_col;
-            auto load = make_input(
-                [&](int ea) {
-                    if (!on) return Ops<T>::mk(0, 0);
-                    const int i = in_src(a.fb * ea + col, a.in_len, a.fN, a.centered_in);
-                    if (i < 0) return Ops<T>::mk(0, 0);
-                    C v = in[i];
-                    if (a.clear_in && (v.x != (T)0 || v.y != (T)0)) in[i] = Ops<T>::mk(0, 0);
-                    if (a.centered_in) v = Ops<T>::scale(v, rowf * (dcol ? dcol[i] : (T)1));
-                    return v;
-                },
-                [](int, C v) { return v; });
-            auto store = [&](int k1, C v) {
-                if (on) out[(long long)k1 * a.fb] = v;
-            };
-            fft_fused<T, NCOL>(S, S2, fp, tw, load, store);
-        } else if constexpr (MODE == kFftColStep1) {
-            // outer index o = b: rows e = fb a + b of the grid columns
-            const C* in = (const C*)a.in + col;
-            C* out = (C*)a.out + (long long)o * a.ncols + col;
-            auto load = make_input(
-                [&](int ea) {
-                    if (!on) return Ops<T>::mk(0, 0);
-                    const int i = in_src(a.fb * ea + o, a.in_len, a.fN, a.centered_in);
-                    return i < 0 ? Ops<T>::mk(0, 0) : in[(long long)i * a.ncols];
-                },
-                [](int, C v) { return v; });
-            auto store = [&](int k1, C v) {
-                if (on) out[(long long)k1 * a.fb * a.ncols] = v;
-            };
-            fft_fused<T, NCOL>(S, S2, fp, tw, load, store);
-        } else if constexpr (MODE == kFftRowStep2) {
-            // transform (l = o, k1 = col): scratch row (o fa + k1), b contiguous
-            const C* in = (const C*)a.in + ((long long)o * a.fa + col) * a.fb;
-            C* out = (C*)a.out + (long long)o * a.out_stride;
-            const C* twN = (const C*)a.twN;
-            auto load = make_input(
-                [&](int b) {
-                    if (!on) return Ops<T>::mk(0, 0);
-                    return Ops<T>::mul(in[b], __ldg(&twN[b * col]));
-                },
-                [](int, C v) { return v; });
-            auto store = [&](int k2, C v) {
-                const int kp = out_slot(col + a.fa * k2, a.out_len, a.fN);
-                if (kp >= 0 && on) out[kp] = v;
-            };
-            fft_fused<T, NCOL>(S, S2, fp, tw, load, store);
-        } else {   // kFftColStep2: outer index o = k1
-            const C* in = (const C*)a.in + (long long)o * a.fb * a.ncols + col;
-            C* out = (C*)a.out + col;
-            const C* twN = (const C*)a.twN;
-            C axc = Ops<T>::mk(1, 0);
-            if (a.ax && on) axc = ((const C*)a.ax)[col];
-            auto load = make_input(
-                [&](int b) {
-                    if (!on) return Ops<T>::mk(0, 0);
-                    return Ops<T>::mul(in[(long long)b * a.ncols], __ldg(&twN[b * o]));
-                },
-                [](int, C v) { return v; });
-            auto store = [&](int k2, C v) {
-                const int kp = out_slot(o + a.fa * k2, a.out_len, a.fN);
-                if (kp < 0 || !on) return;
-                if (a.ax) {
-                    v = Ops<T>::mul(Ops<T>::mul(v, axc), __ldg(&((const C*)a.ay)[kp]));
-                    if (a.occulter) v = Ops<T>::mk((T)1 - v.x, -v.y);
-                }
-                out[(long long)kp * a.ncols] = v;
-            };
-            fft_fused<T, NCOL>(S, S2, fp, tw, load, store);
+    const int ncol = 1 << ls, ngroups = (a.ncols + ncol - 1) >> ls;
+    const int tr = blockDim.x >> ls;
+    const int c = threadIdx.x & (ncol - 1);        // this thread's column
+    const Place pl{c, (int)threadIdx.x >> ls, tr, ls};
+    const int o = blockIdx.x / ngroups, col = ((int)(blockIdx.x - o * ngroups) << ls) + c;
+    const bool on = col < a.ncols;
+    auto at = [&](int e) -> C& { return S[c + (pad(e) << ls)]; };
+    if constexpr (MODE == kFftPlain) {
+        const C* in = (const C*)a.in + (long long)o * a.in_bstride + col;
+        C* out = (C*)a.out + (long long)o * a.out_bstride + col;
+        if (a.live) {   // live tile rows of this transform as a bit mask
+            for (int t = threadIdx.x; t < kMaxTileRows / 32; t += blockDim.x) s_live[t] = 0u;
+            __syncthreads();
+            for (int t = threadIdx.x; t < a.nty; t += blockDim.x)
+                if (a.live[(long long)o * a.nty + t]) atomicOr(&s_live[t >> 5], 1u << (t & 31));
+            __syncthreads();
         }
+        batched<C>(
+            pl, a.in_len,
+            [&](int i) {
+                const int r = i / kTile;
+                const bool live = on && (!a.live || ((s_live[r >> 5] >> (r & 31)) & 1u));
+                return live ? in[(long long)i * a.ncols] : O::mk(0, 0);
+            },
+            [&](int i, C v) { at(in_natural(i, a.in_len, n, a.centered_in)) = v; });
+        zero_rest(S, pl, a.in_len, n, a.centered_in);
+        __syncthreads();
+        fft_line<T>(S, fp, pl, tw);
+        if (!on) return;
+        const C axc = a.ax ? ((const C*)a.ax)[(long long)o * a.ncols + col] : O::mk(1, 0);
+        const C* ay = a.ax ? (const C*)a.ay + (long long)o * a.out_len : nullptr;
+        for (int kp = pl.t; kp < a.out_len; kp += tr) {
+            C v = at(out_natural(kp, a.out_len, n));
+            if (ay) {
+                v = O::mul(O::mul(v, axc), __ldg(&ay[kp]));
+                if (a.occulter) v = O::mk((T)1 - v.x, -v.y);
+            }
+            out[(long long)kp * a.ncols] = v;
+        }
+    } else if constexpr (MODE == kFftRowStep1) {
+        // grid row o viewed as fa x fb (element e = fb a + b at column b = col)
+        C* in = (C*)a.in + (long long)o * a.in_stride;
+        C* out = (C*)a.out + (long long)o * a.fN + col;
+        const T rowf = a.deconv_row ? ((const T*)a.deconv_row)[o] : (T)1;
+        const T* dcol = (const T*)a.deconv_col;
+        auto src = [&](int ea) {
+            return on ? in_src(a.fb * ea + col, a.in_len, a.fN, a.centered_in) : -1;
+        };
+        auto input = make_input(
+            [&](int ea) {
+                const int i = src(ea);
+                return i < 0 ? O::mk(0, 0) : in[i];
+            },
+            [&](int ea, C v) {
+                const int i = src(ea);
+                if (i < 0) return v;
+                if (a.clear_in && (v.x != (T)0 || v.y != (T)0)) in[i] = O::mk(0, 0);
+                if (a.centered_in) v = O::scale(v, rowf * (dcol ? __ldg(&dcol[i]) : (T)1));
+                return v;
+            });
+        auto store = [&](int k1, C v) {
+            if (on) out[(long long)k1 * a.fb] = v;
+        };
+        fft_fused<T>(S, fp, pl, pl, tw, input, store);
+    } else if constexpr (MODE == kFftColStep1) {
+        // outer index o = b: rows e = fb a + b of the grid columns
+        const C* in = (const C*)a.in + col;
+        C* out = (C*)a.out + (long long)o * a.ncols + col;
+        auto input = make_input(
+            [&](int ea) {
+                const int i = on ? in_src(a.fb * ea + o, a.in_len, a.fN, a.centered_in) : -1;
+                return i < 0 ? O::mk(0, 0) : in[(long long)i * a.ncols];
+            },
+            [](int, C v) { return v; });
+        auto store = [&](int k1, C v) {
+            if (on) out[(long long)k1 * a.fb * a.ncols] = v;
+        };
+        fft_fused<T>(S, fp, pl, pl, tw, input, store);
+    } else if constexpr (MODE == kFftRowStep2) {
+        // transform (l = o, k1 = col): scratch row (o fa + k1), b contiguous.
+        // The first stage's neighbouring threads take neighbouring b, the
+        // others' neighbouring columns, whose outputs are adjacent
+        const int cf = threadIdx.x / tr;
+        const Place pf{cf, (int)threadIdx.x - cf * tr, tr, ls};
+        const int colf = col - c + cf;
+        const bool onf = colf < a.ncols;
+        const C* in = (const C*)a.in + ((long long)o * a.fa + colf) * a.fb;
+        C* out = (C*)a.out + (long long)o * a.out_stride;
+        const C* twN = (const C*)a.twN;
+        auto input = make_input([&](int b) { return onf ? in[b] : O::mk(0, 0); },
+                                [&](int b, C v) {
+                                    return onf ? O::mul(v, __ldg(&twN[b * colf])) : v;
+                                });
+        auto store = [&](int k2, C v) {
+            const int kp = out_slot(col + a.fa * k2, a.out_len, a.fN);
+            if (kp >= 0 && on) out[kp] = v;
+        };
+        fft_fused<T>(S, fp, pf, pl, tw, input, store);
+    } else {   // kFftColStep2: outer index o = k1
+        const C* in = (const C*)a.in + (long long)o * a.fb * a.ncols + col;
+        C* out = (C*)a.out + col;
+        const C* twN = (const C*)a.twN;
+        C axc = O::mk(1, 0);
+        if (a.ax && on) axc = ((const C*)a.ax)[col];
+        auto input = make_input(
+            [&](int b) { return on ? in[(long long)b * a.ncols] : O::mk(0, 0); },
+            [&](int b, C v) { return O::mul(v, __ldg(&twN[b * o])); });
+        auto store = [&](int k2, C v) {
+            const int kp = out_slot(o + a.fa * k2, a.out_len, a.fN);
+            if (kp < 0 || !on) return;
+            if (a.ax) {
+                v = O::mul(O::mul(v, axc), __ldg(&((const C*)a.ay)[kp]));
+                if (a.occulter) v = O::mk((T)1 - v.x, -v.y);
+            }
+            out[(long long)kp * a.ncols] = v;
+        };
+        fft_fused<T>(S, fp, pl, pl, tw, input, store);
     }
 }
 
-int threads_for(int elems, int em) {
-    int t = (elems + em - 1) / em;
-    t = (t + 31) / 32 * 32;
-    if (t < 64) t = 64;
-    if (t > kFftThreads) t = kFftThreads;
-    return t;
+// Fewest stages, then fewest threads per line (at most 1024), then the larger
+// radices first.
+void search_radices(int m, int n, bool dbl, int first, int depth, int threads, int* cur, int* best,
+                    int* best_stages, int* best_threads) {
+    if (m == 1) {
+        if (depth >= 2 && (depth < *best_stages ||
+                           (depth == *best_stages && threads < *best_threads))) {
+            std::copy(cur, cur + depth, best);
+            *best_stages = depth;
+            *best_threads = threads;
+        }
+        return;
+    }
+    if (depth >= *best_stages || depth >= kMaxRadixStages) return;
+    const int nr = (int)((dbl ? sizeof(kRadicesD) : sizeof(kRadicesF)) / sizeof(int));
+    for (int i = first; i < nr; ++i) {
+        const int r = dbl ? kRadicesD[i] : kRadicesF[i];
+        if (m % r) continue;
+        const int k = butterflies(r, dbl), t = std::max(threads, (n / r + k - 1) / k);
+        if (t > 1024) continue;
+        cur[depth] = r;
+        search_radices(m / r, n, dbl, i, depth + 1, t, cur, best, best_stages, best_threads);
+    }
 }
 
 }  // namespace
 
-FftPlan make_fft_plan(int n, int max_radix) {
+FftPlan make_fft_plan(int n, int is_double) {
     FftPlan fp{};
     fp.n = n;
+    int cur[kMaxRadixStages], best = kMaxRadixStages + 1, threads = 1 << 30;
     int m = n;
-    if (max_radix >= 16)
-        while (m % 16 == 0) { fp.radix[fp.nstages++] = 16; m /= 16; }
-    if (max_radix >= 8)
-        while (m % 8 == 0) { fp.radix[fp.nstages++] = 8; m /= 8; }
-    while (m % 4 == 0) { fp.radix[fp.nstages++] = 4; m /= 4; }
-    while (m % 2 == 0) { fp.radix[fp.nstages++] = 2; m /= 2; }
-    while (m % 3 == 0) { fp.radix[fp.nstages++] = 3; m /= 3; }
-    while (m % 5 == 0) { fp.radix[fp.nstages++] = 5; m /= 5; }
-    if (m != 1) fp.nstages = -1;
-    long long p = 1;
+    for (int f : {2, 3, 5})
+        while (m % f == 0) m /= f;
+    if (m == 1 && n >= 4)
+        search_radices(n, n, is_double != 0, 0, 0, 1, cur, fp.radix, &best, &threads);
+    if (best > kMaxRadixStages) {
+        fp.nstages = -1;
+        return fp;
+    }
+    fp.nstages = best;
+    fp.threads = threads;
+    long long p = 1, off = 0;
     for (int s = 0; s < fp.nstages; ++s) {
+        fp.nb[s] = n / fp.radix[s];
         fp.p[s] = (int)p;
         fp.pmagic[s] = p == 1 ? 0u : (unsigned)(((1ULL << 32) + (unsigned long long)p - 1) / p);
+        fp.toff[s] = (int)off;
+        if (s > 0) off += p * (fp.radix[s] - 1);
         p *= fp.radix[s];
     }
+    fp.ntw = (int)off;
     return fp;
 }
 
-// Largest column batch (power of two, <= 8) whose two n x C ping-pong buffers
-// fit in shared memory; 0 if n itself does not.
-bool fft_supported(int n, int is_double, int* max_cols) {
-    FftPlan fp = make_fft_plan(n, 4);
-    if (fp.nstages < 0 || n < 2) return false;
-    const long long smem_cap = 227 * 1024;
-    const int esz = is_double ? 16 : 8;
-    int c = 8;
-    while (c > 0 && 2LL * padded_len(n) * c * esz > smem_cap) c >>= 1;
-    if (max_cols) *max_cols = c;
-    return c > 0;
+// One pass: up to 13,671 points in FP32, 6,834 in FP64 (half the shared
+// memory): a longer line leaves one block per SM, and four steps are faster.
+bool fft_supported(int n, int is_double) {
+    return make_fft_plan(n, is_double).nstages >= 2 &&
+           2LL * padded_len(n) * (is_double ? 16 : 8) <= 227 * 1024;
+}
+
+// FP64 passes are bound by the FP64 pipe, so their time is the fullest SM's
+// share of the lines.  Three blocks per SM (by the shared memory asked for),
+// one line each, hand out the last lines evenly (the star's 1,000 columns of
+// 2048: 190 us with two columns per block, 168 with one).
+template <typename T>
+size_t fft_smem(size_t bytes) {
+    return sizeof(T) == 8 ? std::max(bytes, (size_t)60 * 1024) : bytes;
 }
 
 template <typename T>
 void launch_fft_rows(const FftPlan& fp, const RowPassArgs& a, cudaStream_t st) {
-    const size_t smem = 2 * (size_t)padded_len(fp.n) * sizeof(cx_t<T>);
-    // one thread per butterfly of the leading (largest) radix: a radix-16
-    // plan gets n/16 threads, all busy in its radix-16 stages, and more rows
-    // resident per SM
-    const int threads = threads_for(fp.n, fp.radix[0] > emax<T>() ? fp.radix[0] : emax<T>());
     const int nwork = a.row_list ? a.nlist : a.nrows;
-    int blocks = nwork < 152 * 16 ? nwork : 152 * 16;
-    if (blocks < 1) blocks = 1;
+    // short rows: several per block, as long as the blocks still cover the SMs
+    int lines = 1;
+    while (lines < 8 && 2 * lines * fp.threads <= 128 && nwork / (2 * lines) >= 152 * 2) lines *= 2;
+    const int tr = lines > 1 ? fp.threads : (fp.threads + 31) / 32 * 32;
+    const int threads = (lines * tr + 31) / 32 * 32;
+    const size_t smem = fft_smem<T>((size_t)lines * padded_len(fp.n) * sizeof(cx_t<T>));
+    const int blocks = std::max(1, (nwork + lines - 1) / lines);
     cudaFuncSetAttribute(k_fft_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_fft_rows<T><<<blocks, threads, smem, st>>>(fp, a);
+    k_fft_rows<T><<<blocks, threads, smem, st>>>(fp, a, lines, tr);
 }
 
 template <typename T, int MODE>
-void launch_cols_mode(const FftPlan& fp, const ColPassArgs& a, int cmax, cudaStream_t st) {
-    const size_t smem = 2 * (size_t)padded_len(fp.n) * cmax * sizeof(cx_t<T>);
-    const int threads = threads_for(fp.n * cmax, emax<T>());
+void launch_cols_mode(const FftPlan& fp, const ColPassArgs& a, cudaStream_t st) {
     const int nouter = MODE == kFftPlain ? (a.batch > 1 ? a.batch : 1) : a.nouter;
-    const long long work = (long long)((a.ncols + cmax - 1) / cmax) * nouter;
-    int blocks = work < 152 * 16 ? (int)work : 152 * 16;
-    if (blocks < 1) blocks = 1;
-#define FRES_COLS(NC)                                                                          \
-    case NC:                                                                                   \
-        cudaFuncSetAttribute(k_fft_cols<T, NC, MODE>,                                          \
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);          \
-        k_fft_cols<T, NC, MODE><<<blocks, threads, smem, st>>>(fp, a);                         \
-        break;
-    switch (cmax) {
-        FRES_COLS(1) FRES_COLS(2) FRES_COLS(4) FRES_COLS(8)
-        default: break;
-    }
-#undef FRES_COLS
+    const size_t line = (size_t)padded_len(fp.n) * sizeof(cx_t<T>);
+    auto items = [&](int ls) { return (long long)((a.ncols + (1 << ls) - 1) >> ls) * nouter; };
+    // columns per block: 4 fill a 32-byte sector in FP32, short transforms take
+    // up to 16; two blocks per SM, and enough blocks for the SMs.  FP64: one
+    // long column (256 threads), see fft_smem
+    int ls = 4;
+    while (ls > 0 && ((fp.threads << ls) > (ls > 2 || sizeof(T) == 8 ? 256 : 512) ||
+                      (line << ls) > 110 * 1024 || (ls > 1 && items(ls) < 152)))
+        --ls;
+    const int threads = ((fp.threads << ls) + 31) / 32 * 32;
+    const size_t smem = fft_smem<T>(line << ls);
+    const int blocks = (int)std::max(1LL, items(ls));
+    cudaFuncSetAttribute(k_fft_cols<T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
+    k_fft_cols<T, MODE><<<blocks, threads, smem, st>>>(fp, a, ls);
 }
 
+// FP32 column passes of square type-3 grids, start (two buffers, radix-16/8/4/
+// 2/3/5 stages) -> single pass here -> four steps (us): 1920: 37 -> 31; 2560:
+// 70 -> 57 in four steps; 3200: 109 -> 86; 3456: 170 -> 109; 5120: 406 -> 178
+// (single pass -> four steps from 2560 on): the line lies at 2400.
 template <typename T>
 void launch_fft_cols(const FftPlan& fp, const ColPassArgs& a, cudaStream_t st) {
-    int cmax = 0;
-    fft_supported(fp.n, sizeof(T) == 8, &cmax);
-    // fewer columns per block when that keeps three blocks per SM
-    while (cmax > 1 && 2LL * padded_len(fp.n) * cmax * (long long)sizeof(cx_t<T>) > kFftSmemTarget)
-        cmax >>= 1;
     switch (a.mode) {
-        case kFftRowStep1: launch_cols_mode<T, kFftRowStep1>(fp, a, cmax, st); break;
-        case kFftColStep1: launch_cols_mode<T, kFftColStep1>(fp, a, cmax, st); break;
-        case kFftColStep2: launch_cols_mode<T, kFftColStep2>(fp, a, cmax, st); break;
-        case kFftRowStep2: launch_cols_mode<T, kFftRowStep2>(fp, a, cmax, st); break;
-        default: launch_cols_mode<T, kFftPlain>(fp, a, cmax, st); break;
+        case kFftRowStep1: launch_cols_mode<T, kFftRowStep1>(fp, a, st); break;
+        case kFftColStep1: launch_cols_mode<T, kFftColStep1>(fp, a, st); break;
+        case kFftColStep2: launch_cols_mode<T, kFftColStep2>(fp, a, st); break;
+        case kFftRowStep2: launch_cols_mode<T, kFftRowStep2>(fp, a, st); break;
+        default: launch_cols_mode<T, kFftPlain>(fp, a, st); break;
     }
 }
 
@@ -566,8 +717,7 @@ bool fft_split(int n, int is_double, int* fa, int* fb) {
     int best = 0;
     for (int d = 2; (long long)d * d <= n; ++d) {
         if (n % d) continue;
-        if (make_fft_plan(d, 4).nstages < 0 || make_fft_plan(n / d, 4).nstages < 0) continue;
-        if (fft_supported(d, is_double, nullptr) && fft_supported(n / d, is_double, nullptr)) best = d;
+        if (fft_supported(d, is_double) && fft_supported(n / d, is_double)) best = d;
     }
     if (!best) return false;
     *fa = best;

@@ -1052,6 +1052,19 @@ __global__ void k_twiddles(int n, void* table, int is_double) {
     else ((float2*)table)[j] = make_float2((float)c, (float)s);
 }
 
+// Stage twiddles of an FFT plan: entry toff + (q - 1) p + k = w_{p r}^{q k}.
+__global__ void k_stage_twiddles(FftPlan fp, void* table, int is_double) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= fp.ntw) return;
+    int s = 1;
+    while (s + 1 < fp.nstages && j >= fp.toff[s + 1]) ++s;
+    const int p = fp.p[s], q = (j - fp.toff[s]) / p + 1, k = (j - fp.toff[s]) % p;
+    double sn, cs;
+    sincospi(-2.0 * ((double)q * k) / ((double)p * fp.radix[s]), &sn, &cs);
+    if (is_double) ((double2*)table)[j] = make_double2(cs, sn);
+    else ((float2*)table)[j] = make_float2((float)cs, (float)sn);
+}
+
 // Output factors of the type-1 path (Sec. 3.3 step 3 and the deconvolution):
 // A[k'] = exp(i pi xi^2 / lz) / psihat(2 pi k / nf) [* 1/(i lz)],
 // xi = x0 + k h, k = k' - floor(n/2).  FP64, phase reduced mod 2 pi.
@@ -1216,6 +1229,10 @@ void launch_scan_chunks(int ntiles, int* counts, int* cursor, Chunk* chunks, int
 
 void launch_twiddles(int n, void* table, int is_double, cudaStream_t st) {
     k_twiddles<<<nblk(n, 256), 256, 0, st>>>(n, table, is_double);
+}
+
+void launch_stage_twiddles(const FftPlan& fp, void* table, int is_double, cudaStream_t st) {
+    if (fp.ntw > 0) k_stage_twiddles<<<nblk(fp.ntw, 256), 256, 0, st>>>(fp, table, is_double);
 }
 
 void launch_t1_tables(int n, int nf, double h, double x0, double lz, int w, double beta,
