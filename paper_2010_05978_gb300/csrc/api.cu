@@ -108,6 +108,8 @@ struct Plan {
     FftDim d1{}, d2{};            // FFT along x (rows) and y (columns)
     void* fscratch = nullptr;     // four-step intermediate
     std::vector<void*> allocs;
+    char* slab = nullptr;         // small allocations are carved from 1 MB slabs (in allocs)
+    size_t slab_left = 0;
     long long bytes = 0;
     void* rec = nullptr;
     void* sorted = nullptr;
@@ -196,12 +198,31 @@ fresnel_status dalloc(Plan* p, void** out, size_t bytes) {
     if (p->opts.max_device_bytes > 0 && p->bytes + (long long)bytes > p->opts.max_device_bytes)
         return fres_fail(FRESNEL_ERR_OOM, "plan would exceed max_device_bytes (" +
                                                std::to_string(p->opts.max_device_bytes) + ")");
-    cudaError_t e = cudaMalloc(out, bytes);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return fres_fail(FRESNEL_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    // A plan holds a dozen small tables per family: carved from slabs they cost
+    // one cudaMalloc and cudaFree per megabyte (an eight-wavelength starshade
+    // plan: 240 -> 20 of each).  Under a memory cap every allocation is its own,
+    // so that the cap counts all that is held.
+    constexpr size_t kSlab = 1 << 20, kSmall = 64 << 10;
+    const bool small = bytes <= kSmall && p->opts.max_device_bytes == 0;
+    const size_t carve = (bytes + 255) & ~(size_t)255;
+    if (!small || p->slab_left < carve) {
+        cudaError_t e = cudaMalloc(out, small ? kSlab : bytes);
+        if (e != cudaSuccess) {
+            *out = nullptr;
+            cudaGetLastError();
+            return fres_fail(FRESNEL_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+        }
+        p->allocs.push_back(*out);
+        if (small) {
+            p->slab = (char*)*out;
+            p->slab_left = kSlab;
+        }
     }
-    p->allocs.push_back(*out);
+    if (small) {
+        *out = p->slab;
+        p->slab += carve;
+        p->slab_left -= carve;
+    }
     p->bytes += (long long)bytes;
     return FRESNEL_OK;
 }
@@ -303,20 +324,22 @@ void choose_kernel(Plan* p) {
 // grows until the maximum error (on a fine grid) stops improving or drops
 // below `stop`; the kernel's square-root end points set a floor near
 // beta e^-beta / deg.  Returns the kept table's maximum error.
-template <typename Tab, typename R, int kMaxDeg>
+// The coefficients are formed in long double, which is software quad
+// precision on some hosts, so nothing is evaluated twice: the kernel once per
+// interpolation point, the cosines once per degree.  The error grid (Err)
+// only chooses the degree: double resolves an FP32 table's errors (>= 1e-9).
+template <typename Tab, typename R, int kMaxDeg, typename Err>
 double fit_pieces(int w, double beta, int deg0, double stop, Tab* h) {
-    auto psi = [&](long double z) -> long double {
-        long double a = 1.0L - z * z;
-        return a > 0 ? std::exp((long double)beta * (std::sqrt(a) - 1.0L)) : 0.0L;
-    };
-    // the kernel on each piece's error grid, once for every degree tried
-    // (long double is software quad precision on some hosts)
+    const int pieces = (w + 1) / 2;
     constexpr int kGrid = 400;
-    std::vector<long double> gv((size_t)((w + 1) / 2) * (kGrid + 1));
-    for (int a = 0; a < (w + 1) / 2; ++a)
+    std::vector<Err> gt(kGrid + 1), gv((size_t)pieces * (kGrid + 1));
+    for (int i = 0; i <= kGrid; ++i) gt[i] = (Err)-1 + i / ((Err)0.5 * kGrid);
+    for (int a = 0; a < pieces; ++a)
         for (int i = 0; i <= kGrid; ++i) {
-            const long double f = 0.5L * (-1.0L + i / (0.5L * kGrid) + 1.0L);
-            gv[(size_t)a * (kGrid + 1) + i] = psi(((long double)a + 1.0L - 0.5L * w - f) * 2.0L / w);
+            const Err f = (Err)0.5 * (gt[i] + (Err)1);
+            const Err z = ((Err)a + (Err)1 - (Err)0.5 * w - f) * (Err)2 / w;
+            const Err r = (Err)1 - z * z;
+            gv[(size_t)a * (kGrid + 1) + i] = r > 0 ? std::exp((Err)beta * (std::sqrt(r) - (Err)1)) : (Err)0;
         }
     double prev_err = 1e300, best_err = 1e300;
     Tab best{};
@@ -326,18 +349,23 @@ double fit_pieces(int w, double beta, int deg0, double stop, Tab* h) {
         Tab t{};
         t.deg = d;
         double err = 0.0;
-        for (int a = 0; a < (w + 1) / 2; ++a) {
-            auto g = [&](long double tt) {
-                long double f = 0.5L * (tt + 1.0L);
-                return psi(((long double)a + 1.0L - 0.5L * w - f) * 2.0L / w);
-            };
+        std::vector<long double> x(n), ck((size_t)n * n), g(n);   // points, cos(k th_i), kernel
+        for (int i = 0; i < n; ++i) {
+            const long double th = 3.14159265358979323846264338327950288L * (i + 0.5L) / n;
+            x[i] = std::cos(th);
+            for (int k = 0; k < n; ++k) ck[(size_t)k * n + i] = std::cos(k * th);
+        }
+        for (int a = 0; a < pieces; ++a) {
+            for (int i = 0; i < n; ++i) {
+                const long double f = 0.5L * (x[i] + 1.0L);
+                const long double z = ((long double)a + 1.0L - 0.5L * w - f) * 2.0L / w;
+                const long double r = 1.0L - z * z;
+                g[i] = r > 0 ? std::exp((long double)beta * (std::sqrt(r) - 1.0L)) : 0.0L;
+            }
             std::vector<long double> b(n), mono(n, 0.0L), T0(n, 0.0L), T1(n, 0.0L), T2(n);
             for (int k = 0; k < n; ++k) {
                 long double acc = 0.0L;
-                for (int i = 0; i < n; ++i) {
-                    long double th = 3.14159265358979323846264338327950288L * (i + 0.5L) / n;
-                    acc += g(std::cos(th)) * std::cos(k * th);
-                }
+                for (int i = 0; i < n; ++i) acc += g[i] * ck[(size_t)k * n + i];
                 b[k] = (k == 0 ? 1.0L : 2.0L) * acc / n;
             }
             T0[0] = 1.0L;
@@ -351,13 +379,15 @@ double fit_pieces(int w, double beta, int deg0, double stop, Tab* h) {
                     T1 = T2;
                 }
             }
+            std::vector<Err> m(n);
             for (int j = 0; j < n; ++j) {
                 if (j % 2 == 0) t.e[a][j / 2] = (R)mono[j];
                 else t.o[a][j / 2] = (R)mono[j];
+                m[j] = (Err)mono[j];
             }
             for (int i = 0; i <= kGrid; ++i) {
-                long double tt = -1.0L + i / (0.5L * kGrid), acc = 0.0L;
-                for (int j = n - 1; j >= 0; --j) acc = acc * tt + mono[j];
+                Err acc = 0;
+                for (int j = n - 1; j >= 0; --j) acc = acc * gt[i] + m[j];
                 err = std::max(err, (double)std::fabs(acc - gv[(size_t)a * (kGrid + 1) + i]));
             }
         }
@@ -373,11 +403,11 @@ double fit_pieces(int w, double beta, int deg0, double stop, Tab* h) {
 }
 
 void fit_horner(int w, double beta, HornerTab* h) {
-    fit_pieces<HornerTab, float, kHornerDeg>(w, beta, 4, 1e-9, h);
+    fit_pieces<HornerTab, float, kHornerDeg, double>(w, beta, 4, 1e-9, h);
 }
 
 double fit_horner_d(int w, double beta, HornerTabD* h) {
-    return fit_pieces<HornerTabD, double, kHornerDegD>(w, beta, 6, 1e-16, h);
+    return fit_pieces<HornerTabD, double, kHornerDegD, long double>(w, beta, 6, 1e-16, h);
 }
 
 fresnel_status validate_family(const fresnel_family& f, long long* n_bdry, long long* n_nodes,
@@ -1575,14 +1605,14 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
         FRES_TRY(dalloc(p, &p->inter, cs * (size_t)p->nf2 * p->n1 * p->B));
         FRES_TRY(dalloc(p, &p->ax, cs * p->n1 * p->B));
         FRES_TRY(dalloc(p, &p->ay, cs * p->n2 * p->B));
-        for (int b = 0; b < p->B; ++b) {   // per problem: the chirp depends on lambda z
-            launch_t1_tables(p->n1, p->nf1, p->opts.grid_h, p->opts.grid_x0, p->lzs[b], w,
-                             p->ks.beta, 1, p->cps[b].sh1, (char*)p->ax + cs * p->n1 * b, dbl,
-                             p->gq_t, p->gq_w, p->gq_n, p->st);
-            launch_t1_tables(p->n2, p->nf2, p->opts.grid_h, p->opts.grid_y0, p->lzs[b], w,
-                             p->ks.beta, 0, p->cps[b].sh2, (char*)p->ay + cs * p->n2 * b, dbl,
-                             p->gq_t, p->gq_w, p->gq_n, p->st);
-        }
+        // per problem: the chirp depends on lambda z
+        double* d_lz = nullptr;
+        FRES_TRY(dalloc(p, (void**)&d_lz, sizeof(double) * p->B));
+        FRES_CK(cudaMemcpyAsync(d_lz, p->lzs.data(), sizeof(double) * p->B, cudaMemcpyHostToDevice, p->st));
+        launch_t1_tables(p->B, d_lz, p->n1, p->nf1, p->opts.grid_h, p->opts.grid_x0, w, p->ks.beta, 1,
+                         p->cps[0].sh1, p->ax, dbl, p->gq_t, p->gq_w, p->gq_n, p->st);
+        launch_t1_tables(p->B, d_lz, p->n2, p->nf2, p->opts.grid_h, p->opts.grid_y0, w, p->ks.beta, 0,
+                         p->cps[0].sh2, p->ay, dbl, p->gq_t, p->gq_w, p->gq_n, p->st);
     } else {
         FRES_TRY(dalloc(p, &p->inter, cs * (size_t)p->nf2 * p->nfft1));
         FRES_TRY(dalloc(p, &p->F, cs * (size_t)p->nfft2 * p->nfft1));

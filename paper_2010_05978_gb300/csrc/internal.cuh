@@ -360,7 +360,8 @@ void launch_twiddles(int n, void* table, int is_double, cudaStream_t st);
 void launch_stage_twiddles(const FftPlan& fp, void* table, int is_double, cudaStream_t st);
 // t1 output tables Ax[k1] = chirp(xi)/(i lz)/psihat(k1), Ay[k2] = chirp(eta)/psihat(k2),
 // each times exp(2 pi i k shift / nf) for a grid spread shifted by shift cells
-void launch_t1_tables(int n, int nf, double h, double x0, double lz, int w, double beta,
+// (B tables of n, one per problem's lz)
+void launch_t1_tables(int B, const double* lz, int n, int nf, double h, double x0, int w, double beta,
                       int with_ilz, int shift, void* table, int is_double, const double* gq_t,
                       const double* gq_w, int q, cudaStream_t st);
 // t3 type-2 deconvolution factors 1/psihat(2 pi l / nfft), l in [-ng/2, ng/2)

@@ -1068,11 +1068,14 @@ __global__ void k_stage_twiddles(FftPlan fp, void* table, int is_double) {
 // Output factors of the type-1 path (Sec. 3.3 step 3 and the deconvolution):
 // A[k'] = exp(i pi xi^2 / lz) / psihat(2 pi k / nf) [* 1/(i lz)],
 // xi = x0 + k h, k = k' - floor(n/2).  FP64, phase reduced mod 2 pi.
-__global__ void k_t1_tables(int n, int nf, double h, double x0, double lz, int w, double beta,
+// Block row b: problem b's table.
+__global__ void k_t1_tables(const double* lzs, int n, int nf, double h, double x0, int w, double beta,
                             int with_ilz, int shift, void* table, int is_double,
                             const double* gq_t, const double* gq_w, int q) {
     int kp = blockIdx.x * blockDim.x + threadIdx.x;
     if (kp >= n) return;
+    const double lz = lzs[blockIdx.y];
+    const long long at = (long long)blockIdx.y * n + kp;
     int k = kp - n / 2;
     double xi = x0 + k * h;
     double ph = reduce_phase(kPi * xi * xi / lz);
@@ -1093,8 +1096,8 @@ __global__ void k_t1_tables(int n, int nf, double h, double x0, double lz, int w
         re = r2;
         im = i2;
     }
-    if (is_double) ((double2*)table)[kp] = make_double2(re, im);
-    else ((float2*)table)[kp] = make_float2((float)re, (float)im);
+    if (is_double) ((double2*)table)[at] = make_double2(re, im);
+    else ((float2*)table)[at] = make_float2((float)re, (float)im);
 }
 
 // Type-3 inner type-2 deconvolution: 1 / psihat(2 pi l / nfft), l = i - ng/2.
@@ -1235,11 +1238,15 @@ void launch_stage_twiddles(const FftPlan& fp, void* table, int is_double, cudaSt
     if (fp.ntw > 0) k_stage_twiddles<<<nblk(fp.ntw, 256), 256, 0, st>>>(fp, table, is_double);
 }
 
-void launch_t1_tables(int n, int nf, double h, double x0, double lz, int w, double beta,
+void launch_t1_tables(int B, const double* lz, int n, int nf, double h, double x0, int w, double beta,
                       int with_ilz, int shift, void* table, int is_double, const double* gq_t,
                       const double* gq_w, int q, cudaStream_t st) {
-    k_t1_tables<<<nblk(n, 128), 128, 0, st>>>(n, nf, h, x0, lz, w, beta, with_ilz, shift, table,
-                                              is_double, gq_t, gq_w, q);
+    for (int b0 = 0; b0 < B; b0 += 65535) {   // grid rows per launch
+        const int nb = std::min(B - b0, 65535);
+        k_t1_tables<<<dim3(nblk(n, 128), nb), 128, 0, st>>>(
+            lz + b0, n, nf, h, x0, w, beta, with_ilz, shift,
+            (char*)table + (size_t)b0 * n * (is_double ? 16 : 8), is_double, gq_t, gq_w, q);
+    }
 }
 
 void launch_t3_deconv(int ng, int nfft, int w, double beta, void* table, int is_double,
