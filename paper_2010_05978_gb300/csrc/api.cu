@@ -1800,7 +1800,10 @@ fresnel_status grad_profile_impl(Plan* p, const void* d_gamma, double* d_grad) {
     FRES_TRY(adjoint_grid<T>(p, d_gamma));
     launch_adj_nodes<T>(p->ft, p->node_blocks, p->grid, p->nf1, p->nf2, p->ks, p->contrib, 0, p->st);
     FRES_TRY(adjoint_release(p));
-    launch_adj_reduce(p->ft.fams, p->pf, p->gofs, p->npf, p->contrib, d_grad, p->st);
+    int max_m = 1;
+    for (const FamilyDev& f : p->fams)
+        if (f.kind == FRESNEL_FAMILY_PETALS) max_m = std::max(max_m, f.m);
+    launch_adj_reduce(p->ft.fams, p->pf, p->gofs, p->npf, max_m, p->contrib, d_grad, p->st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return fres_fail(FRESNEL_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(e));

@@ -413,8 +413,10 @@ void launch_adj_prologue(const void* gamma, const void* ax, const void* ay, void
 template <typename T>
 void launch_adj_nodes(const FamTable& ft, int nblocks, const void* bt, int nf1, int nf2,
                       const KernelShape& ks, double* contrib, int mode, cudaStream_t st);
+// PETALS families pf[0..npf) of at most max_m radii; overwrites their first m
+// contributions
 void launch_adj_reduce(const FamilyDev* fams, const int* pf, const long long* gofs, int npf,
-                       const double* contrib, double* grad, cudaStream_t st);
+                       int max_m, double* contrib, double* grad, cudaStream_t st);
 // Fourier families sf[0..nsf): dL/dr_i into rbuf (at bofs[f]), then dL/dp of
 // each family's 1 + 2K coefficients into grad (at gofs[f])
 void launch_adj_shape_reduce(const FamilyDev* fams, const int* sf, int nsf, int max_params,

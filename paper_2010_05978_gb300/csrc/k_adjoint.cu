@@ -83,11 +83,14 @@ __device__ __forceinline__ void node_derivs(const ChirpParams& cp, double x, dou
         const double z1 = ((double)(a + 1) - 0.5 * W - fr1) * (2.0 / W);
         const double z2 = ((double)(a + 1) - 0.5 * W - fr2) * (2.0 / W);
         const double r1 = 1.0 - z1 * z1, r2 = 1.0 - z2 * z2;
-        p1[a] = r1 > 0.0 ? exp(beta * (sqrt(r1) - 1.0)) : 0.0;
-        p2[a] = r2 > 0.0 ? exp(beta * (sqrt(r2) - 1.0)) : 0.0;
-        // psi'(u) = psi * beta * (-z / sqrt(1 - z^2)) * (2 / W); d/dg = -psi'
-        d1[a] = r1 > 0.0 ? p1[a] * beta * z1 / sqrt(r1) * (2.0 / W) : 0.0;
-        d2[a] = r2 > 0.0 ? p2[a] * beta * z2 / sqrt(r2) * (2.0 / W) : 0.0;
+        // psi'(u) = psi * beta * (-z / sqrt(1 - z^2)) * (2 / W); d/dg = -psi'.
+        // One reciprocal root gives sqrt(r) = r / sqrt(r) too: bound by the
+        // FP64 pipe, where a root and a quotient cost as much as an exp
+        const double i1 = r1 > 0.0 ? rsqrt(r1) : 0.0, i2 = r2 > 0.0 ? rsqrt(r2) : 0.0;
+        p1[a] = r1 > 0.0 ? exp(beta * (r1 * i1 - 1.0)) : 0.0;
+        p2[a] = r2 > 0.0 ? exp(beta * (r2 * i2 - 1.0)) : 0.0;
+        d1[a] = p1[a] * (beta * (2.0 / W)) * (z1 * i1);
+        d2[a] = p2[a] * (beta * (2.0 / W)) * (z2 * i2);
     }
     double Fr = 0, Fi = 0, G1r = 0, G1i = 0, G2r = 0, G2i = 0;
     for (int b = 0; b < W; ++b) {
@@ -242,36 +245,61 @@ __global__ void k_adj_modes(const FamilyDev* __restrict__ fams, const int* __res
     }
 }
 
-// One block per PETALS family (list pf): dL/dA_l = sum over petals and angles
-// of the node contributions (one warp per l), then the profile parameters,
-// added by one thread in increasing l (a fixed order: the gradient repeats
-// bit for bit), kL radii at a time.
+// PETALS families (list pf): dL/dA_l = sum over petals and angles of the node
+// contributions, into the family's first m entries of contrib (whose nodes
+// with angle index 0 of petal 0 are read by the same thread before it writes).
+// A block takes 32 radii, coalesced over l; each of its 8 rows of threads sums
+// every eighth (petal, angle), the rows are added in order: a fixed order, so
+// the gradient repeats bit for bit.
+__global__ void k_adj_lsum(const FamilyDev* __restrict__ fams, const int* __restrict__ pf,
+                           double* __restrict__ contrib) {
+    __shared__ double s_part[8][33];
+    const FamilyDev& f = fams[pf[blockIdx.y]];
+    const int tx = threadIdx.x, ty = threadIdx.y, l = blockIdx.x * 32 + tx;
+    const long long nki = (long long)f.n_panels * f.p;      // nodes per radius
+    if (blockIdx.x * 32 >= f.m) return;                     // the same for the whole block
+    double s = 0.0;
+    if (l < f.m)
+        for (long long e = ty; e < nki; e += 8) s += contrib[f.offset + e * f.m + l];
+    s_part[ty][tx] = s;
+    __syncthreads();
+    if (ty == 0 && l < f.m) {
+        for (int r = 1; r < 8; ++r) s += s_part[r][tx];
+        contrib[f.offset + l] = s;
+    }
+}
+
+// One block per PETALS family: the profile parameters from dL/dA_l.  The
+// threads first find each radius's parameters and factors, kL radii at a time,
+// then every thread adds up its own parameters in increasing l.
 __global__ void k_adj_reduce(const FamilyDev* __restrict__ fams, const int* __restrict__ pf,
                              const long long* __restrict__ gofs,
                              const double* __restrict__ contrib, double* __restrict__ grad) {
-    constexpr int kL = 1024;
-    __shared__ double s_l[kL];
+    constexpr int kL = 256;
+    __shared__ double s_val[kL][4];
+    __shared__ int s_idx[kL][4];
     const FamilyDev& f = fams[pf[blockIdx.x]];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const long long nki = (long long)f.n_panels * f.p;      // nodes per radius
     for (int l0 = 0; l0 < f.m; l0 += kL) {
-        const int l1 = min(l0 + kL, f.m);
-        for (int l = l0 + warp; l < l1; l += nw) {
-            double s = 0.0;
-            for (long long e = lane; e < nki; e += 32) s += contrib[f.offset + e * f.m + l];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) s_l[l - l0] = s;
+        const int nl = min(kL, f.m - l0);
+        for (int i = threadIdx.x; i < nl; i += blockDim.x) {
+            const int l = l0 + i;
+            const double r = f.pa + (f.pR - f.pa) * f.gl_m_a[l], g = contrib[f.offset + l];
+            int idx[4];
+            double val[4];
+            const int cnt = petal_profile_grad(f, l, r, idx, val);
+            for (int q = 0; q < 4; ++q) {
+                s_idx[i][q] = q < cnt ? idx[q] : -1;
+                s_val[i][q] = q < cnt ? g * val[q] : 0.0;
+            }
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int l = l0; l < l1; ++l) {
-                const double r = f.pa + (f.pR - f.pa) * f.gl_m_a[l];
-                int idx[4];
-                double val[4];
-                const int cnt = petal_profile_grad(f, l, r, idx, val);
-                for (int q = 0; q < cnt; ++q) grad[gofs[blockIdx.x] + idx[q]] += s_l[l - l0] * val[q];
-            }
+        for (long long j = threadIdx.x; j < f.n_prof; j += blockDim.x) {
+            double acc = grad[gofs[blockIdx.x] + j];
+            for (int i = 0; i < nl; ++i)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (s_idx[i][q] == (int)j) acc += s_val[i][q];
+            grad[gofs[blockIdx.x] + j] = acc;
         }
         __syncthreads();
     }
@@ -317,8 +345,12 @@ template void launch_adj_nodes<double>(const FamTable&, int, const void*, int, i
                                        const KernelShape&, double*, int, cudaStream_t);
 
 void launch_adj_reduce(const FamilyDev* fams, const int* pf, const long long* gofs, int npf,
-                       const double* contrib, double* grad, cudaStream_t st) {
-    if (npf > 0) k_adj_reduce<<<npf, 256, 0, st>>>(fams, pf, gofs, contrib, grad);
+                       int max_m, double* contrib, double* grad, cudaStream_t st) {
+    if (npf <= 0) return;
+    for (int p0 = 0; p0 < npf; p0 += 65535)   // grid rows per launch
+        k_adj_lsum<<<dim3(nblk(max_m, 32), std::min(npf - p0, 65535)), dim3(32, 8), 0, st>>>(
+            fams, pf + p0, contrib);
+    k_adj_reduce<<<npf, 256, 0, st>>>(fams, pf, gofs, contrib, grad);
 }
 
 void launch_adj_shape_reduce(const FamilyDev* fams, const int* sf, int nsf, int max_params,

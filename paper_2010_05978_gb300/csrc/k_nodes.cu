@@ -108,8 +108,9 @@ __device__ __forceinline__ void legendre_pn(int n, double x, const double* inv, 
                                             double* pn1) {
     double p0 = 1.0, p1 = x;
     for (int j = 1; j < n; ++j) {
-        const double q = (2.0 * j + 1.0) * x * p1 - j * p0;
-        const double p2 = kTable ? q * inv[j + 1] : q / (j + 1.0);
+        // (2j + 1)/(j + 1) x and j/(j + 1) are off the chain p0, p1 -> p2
+        const double r = kTable ? inv[j + 1] : 1.0 / (j + 1.0);
+        const double p2 = fma((2.0 * j + 1.0) * r * x, p1, -(j * r) * p0);
         p0 = p1;
         p1 = p2;
     }
@@ -133,13 +134,16 @@ __global__ void k_gauss_legendre(int n, double* t01, double* w01) {
     double x = (1.0 - (nn - 1.0) / (8.0 * nn * nn * nn)) * cos(kPi * (i + 0.75) / (nn + 0.5));
     if (2 * i + 1 == n) x = 0.0;   // odd n: the middle root
     double pn, pn1;
-    int converged = 0;
-    for (int it = 0; it < 100 && converged < 2; ++it) {
+    // Newton squares the error (times x/(1 - x^2), below n^2/5 at the end
+    // roots), so a step below 1e-11 leaves the root exact to rounding: two or
+    // three steps, each a chain of n dependent recurrences, instead of the
+    // four or five until two steps in a row had vanished
+    for (int it = 0; it < 100; ++it) {
         legendre_pn<kTable>(n, x, s_inv, &pn, &pn1);
         const double dp = nn * (x * pn - pn1) / (x * x - 1.0);
         const double dx = pn / dp;
         x -= dx;
-        if (fabs(dx) < 1e-15) ++converged;
+        if (fabs(dx) < 1e-11) break;
     }
     legendre_pn<kTable>(n, x, s_inv, &pn, &pn1);
     const double dp = nn * (x * pn - pn1) / (x * x - 1.0);
