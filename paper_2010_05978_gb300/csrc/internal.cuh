@@ -231,19 +231,30 @@ __device__ __forceinline__ void horner_eval(const HornerTab& h, float f, float* 
         if (W - 1 - a != a) out[W - 1 - a] = fmaf(-t, O, E);
     }
 }
+// FP64: to the fit's own degree (uniform loops: the FP64 pipe runs at 1/58 of
+// the FP32 rate, so the zero-padded terms cost more than the loops; degree 8
+// instead of 14 at w = 10: 100 instead of 160 multiply-adds per node or target).
 template <int W>
 __device__ __forceinline__ void horner_eval(const HornerTabD& h, double f, double* out) {
     const double t = 2.0 * f - 1.0, u = t * t;
+    constexpr int P = (W + 1) / 2;
+    double E[P], O[P];
+    int k = h.deg / 2;
 #pragma unroll
-    for (int a = 0; a < (W + 1) / 2; ++a) {
-        double E = h.e[a][kHornerEvenD - 1];
+    for (int a = 0; a < P; ++a) E[a] = h.e[a][k];
+    for (--k; k >= 0; --k)
 #pragma unroll
-        for (int k = kHornerEvenD - 2; k >= 0; --k) E = fma(E, u, h.e[a][k]);
-        double O = h.o[a][kHornerOddD - 1];
+        for (int a = 0; a < P; ++a) E[a] = fma(E[a], u, h.e[a][k]);
+    k = (h.deg - 1) / 2;
 #pragma unroll
-        for (int k = kHornerOddD - 2; k >= 0; --k) O = fma(O, u, h.o[a][k]);
-        out[a] = fma(t, O, E);
-        if (W - 1 - a != a) out[W - 1 - a] = fma(-t, O, E);
+    for (int a = 0; a < P; ++a) O[a] = h.o[a][k];
+    for (--k; k >= 0; --k)
+#pragma unroll
+        for (int a = 0; a < P; ++a) O[a] = fma(O[a], u, h.o[a][k]);
+#pragma unroll
+    for (int a = 0; a < P; ++a) {
+        out[a] = fma(t, O[a], E[a]);
+        if (W - 1 - a != a) out[W - 1 - a] = fma(-t, O[a], E[a]);
     }
 }
 

@@ -29,14 +29,14 @@ constexpr int kBin = kTargetBin;    // target bins: kBin x kBin cells of F
 template <typename T>
 __device__ __forceinline__ T kernel_ft_cheb(T t, const T* a, int n, T inv_tmax) {
     const T x = t * inv_tmax;
-    const T y = (T)2 * x * x - (T)1;
+    const T y = (T)2 * x * x - (T)1, y2 = y + y;
     T b1 = 0, b2 = 0;
     for (int k = n - 1; k >= 1; --k) {
-        const T b0 = (T)2 * y * b1 - b2 + a[k];
+        const T b0 = fma(y2, b1, a[k] - b2);   // two operations on the (FP64) pipe
         b2 = b1;
         b1 = b0;
     }
-    return y * b1 - b2 + a[0];
+    return fma(y, b1, a[0] - b2);
 }
 
 // Support start (s1, s2) and fractional offsets of a target in the

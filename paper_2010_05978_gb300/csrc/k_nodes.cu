@@ -100,17 +100,18 @@ __device__ __forceinline__ void node_tiles(int s1, int s2, const ChirpParams& cp
 // (j + 1) P_{j+1} = (2j + 1) x P_j - j P_{j-1}, from Tricomi's asymptotic
 // estimate of each root; the weights 2 / ((1 - x^2) P_n'(x)^2); both mapped
 // from (-1, 1) to (0, 1), ascending.  The roots are symmetric (x_{n-1-i} =
-// -x_i): thread i < ceil(n/2) finds root i and writes both.  The recurrence
-// divides by j + 1 through a per-block table of reciprocals (FP64 division is
-// many times the cost of a multiply).
+// -x_i): thread i < ceil(n/2) finds root i and writes both.  The recurrence's
+// factors come from a per-block table (FP64 division is many times the cost of
+// a multiply), which leaves one multiply-add per step on the dependent chain.
 template <bool kTable>
-__device__ __forceinline__ void legendre_pn(int n, double x, const double* inv, double* pn,
+__device__ __forceinline__ void legendre_pn(int n, double x, const double2* c, double* pn,
                                             double* pn1) {
     double p0 = 1.0, p1 = x;
+#pragma unroll 4
     for (int j = 1; j < n; ++j) {
-        // (2j + 1)/(j + 1) x and j/(j + 1) are off the chain p0, p1 -> p2
-        const double r = kTable ? inv[j + 1] : 1.0 / (j + 1.0);
-        const double p2 = fma((2.0 * j + 1.0) * r * x, p1, -(j * r) * p0);
+        // only the multiply-add is on the chain p0, p1 -> p2
+        const double2 k = kTable ? c[j] : make_double2((2.0 * j + 1.0) / (j + 1.0), j / (j + 1.0));
+        const double p2 = fma(k.x * x, p1, -(k.y * p0));
         p0 = p1;
         p1 = p2;
     }
@@ -118,13 +119,16 @@ __device__ __forceinline__ void legendre_pn(int n, double x, const double* inv, 
     *pn1 = p0;
 }
 
-// kTable: the reciprocals 1/j (j <= n) in dynamic shared memory (n small
-// enough); otherwise the recurrence divides.
+// kTable: the factors (2j + 1) / (j + 1), j / (j + 1) in dynamic shared memory
+// (n small enough); otherwise the recurrence divides.
 template <bool kTable>
 __global__ void k_gauss_legendre(int n, double* t01, double* w01) {
-    extern __shared__ double s_inv[];   // s_inv[j] = 1 / j, j = 1 .. n
+    extern __shared__ double2 s_c[];
     if (kTable) {
-        for (int j = threadIdx.x; j <= n; j += blockDim.x) s_inv[j] = j > 0 ? 1.0 / j : 0.0;
+        for (int j = threadIdx.x; j < n; j += blockDim.x) {
+            const double inv = 1.0 / (j + 1.0);
+            s_c[j] = make_double2((2.0 * j + 1.0) * inv, j * inv);
+        }
         __syncthreads();
     }
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -139,13 +143,13 @@ __global__ void k_gauss_legendre(int n, double* t01, double* w01) {
     // three steps, each a chain of n dependent recurrences, instead of the
     // four or five until two steps in a row had vanished
     for (int it = 0; it < 100; ++it) {
-        legendre_pn<kTable>(n, x, s_inv, &pn, &pn1);
+        legendre_pn<kTable>(n, x, s_c, &pn, &pn1);
         const double dp = nn * (x * pn - pn1) / (x * x - 1.0);
         const double dx = pn / dp;
         x -= dx;
         if (fabs(dx) < 1e-11) break;
     }
-    legendre_pn<kTable>(n, x, s_inv, &pn, &pn1);
+    legendre_pn<kTable>(n, x, s_c, &pn, &pn1);
     const double dp = nn * (x * pn - pn1) / (x * x - 1.0);
     const double w = 1.0 / ((1.0 - x * x) * dp * dp);
     t01[i] = 0.5 * (1.0 - x);
@@ -1120,7 +1124,7 @@ inline int nblk(long long n, int b) { return (int)((n + b - 1) / b); }
 }  // namespace
 
 void launch_gauss_legendre(int n, double* t01, double* w01, cudaStream_t st) {
-    const size_t dyn = sizeof(double) * ((size_t)n + 1);
+    const size_t dyn = sizeof(double2) * (size_t)n;
     const int blocks = nblk((n + 1) / 2, 64);
     if (dyn <= 48 * 1024) {
         k_gauss_legendre<true><<<blocks, 64, dyn, st>>>(n, t01, w01);
