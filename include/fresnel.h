@@ -163,8 +163,10 @@ typedef struct {
     long long max_device_bytes; /* cap on the plan's device memory; 0 = no cap */
     /* SCATTERED + FP32_FAST: bucket the targets by 16 x 16 blocks of the FFT
      * grid and interpolate from shared-memory patches (1), gather each target
-     * straight from global memory (-1), or choose (0: bucket when the FFT grid
-     * exceeds 64 MB, i.e. would not stay in L2, and M >= 32768). */
+     * straight from global memory (-1), or choose (0: bucket when the part of
+     * the FFT grid under the box would not stay in L2 and the targets are
+     * dense: grids above 512 MB with at least one target per 32 cells, above
+     * 256 MB with one per 4). */
     int t3_binning;
     /* FFT lengths above this run as four-step transforms fa x fb (two launches
      * per pass through an intermediate buffer) instead of one shared-memory

@@ -42,13 +42,20 @@ namespace {
 
 constexpr uint64_t kMagic = 0x46524553'4e454c31ull;   // "FRESNEL1"
 constexpr int kMaxEvents = 16;
-// FP32 type-3 target binning (kTargetBin x kTargetBin blocks of the FFT grid, interpolation
-// from shared-memory patches) is chosen automatically only when the FFT grid
-// would not stay in L2 and the target set is large.  Measured on the
-// F = 100 star workload (29 MB grid, 1e6 targets): binned 0.18 ms against
-// 0.126 ms for direct gathers from L2, so small grids gather directly.
-constexpr long long kSortTargetsFrom = 32768;
-constexpr long long kBinFromGridBytes = 64LL << 20;
+// FP32 type-3 target binning (kTargetBin x kTargetBin blocks of the FFT grid,
+// interpolation from shared-memory patches), chosen automatically where direct
+// gathers would come from DRAM and the targets are dense enough to pay for the
+// sort.  A target set covers the central 1 / sigma^2 of the grid, so gathers
+// stay in the 129 MB L2 up to grids of some 400 MB.  Measured, direct against
+// binned (us per call, 1.2e6 and 4e6 targets): 82 MB 245 / 340, 381 / 671;
+// 212 MB 447 / 527, 585 / 725; 382 MB 714 / 811, 907 / 961 (equal at ~8e6);
+// 737 MB 1269 / 1411, 1628 / 1538; 2.4 GB 3930 / 4533, 4474 / 4697 (equal at
+// ~6e6).  Hence one target per 4 grid cells above 256 MB, per 32 above 512 MB.
+bool want_binning(long long M, int nfft1, int nfft2) {
+    const long long cells = (long long)nfft1 * nfft2, bytes = cells * 8;
+    if (bytes > 512LL << 20) return M >= cells / 32;
+    return bytes > 256LL << 20 && M >= cells / 4;
+}
 
 // Column transforms longer than this take four steps in FP32 scattered plans
 // (measured: see the table at launch_fft_cols).
@@ -639,10 +646,8 @@ fresnel_status eval_impl(Plan* p, const double* d_targets, long long M, void* d_
     // times are recorded, so that each stage is timed on its own)
     bool binned = false;
     if (p->tkind == FRESNEL_SCATTERED && M > 0 && sizeof(T) == 4) {
-        const long long fbytes = (long long)p->nfft1 * p->nfft2 * (long long)sizeof(cx_t<T>);
         const bool want = p->opts.t3_binning > 0 ||
-                          (p->opts.t3_binning == 0 && M >= kSortTargetsFrom &&
-                           fbytes > kBinFromGridBytes);
+                          (p->opts.t3_binning == 0 && want_binning(M, p->nfft1, p->nfft2));
         binned = want && M < (1LL << 31) && interp_binned_width(p->ks.w);
     }
     T3Sort sort{};
@@ -2227,7 +2232,9 @@ fresnel_status plan_scattered_batch(const fresnel_problem* problems, int n, doub
 // Grows a type-3 plan's target permutation ahead of graph capture (no
 // allocation may happen while the evaluation is being captured).
 fresnel_status ensure_perm(Plan* q, long long M) {
-    if (q->prec != FRESNEL_FP32_FAST || M < kSortTargetsFrom || M <= q->perm_cap) return FRESNEL_OK;
+    const bool want = q->opts.t3_binning > 0 ||
+                      (q->opts.t3_binning == 0 && want_binning(M, q->nfft1, q->nfft2));
+    if (q->prec != FRESNEL_FP32_FAST || !want || M <= q->perm_cap) return FRESNEL_OK;
     FRES_CK(cudaStreamSynchronize(q->st));
     if (q->perm) cudaFree(q->perm);
     q->perm = nullptr;
