@@ -1580,22 +1580,23 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
     // ---------------- grids and tables
     const size_t cs = p->csize();
     FRES_TRY(dalloc(p, &p->grid, cs * (size_t)p->nf1 * p->nf2 * p->B));
-    // strip spreading adds into a zero grid; the row pass leaves it zero
-    if (p->strips) FRES_CK(cudaMemsetAsync(p->grid, 0, cs * (size_t)p->nf1 * p->nf2 * p->B, p->st));
     // kernel-transform quadrature: Gauss-Legendre on (0,1) with 2w + 16 points
     p->gq_n = std::min(64, 2 * w + 16);
     FRES_TRY(dalloc(p, (void**)&p->gq_t, sizeof(double) * p->gq_n));
     FRES_TRY(dalloc(p, (void**)&p->gq_w, sizeof(double) * p->gq_n));
     launch_gauss_legendre(p->gq_n, p->gq_t, p->gq_w, p->st);
     for (FftDim* d : {&p->d1, &p->d2}) {
-        FRES_TRY(dalloc(p, &d->tw, cs * d->n));
-        launch_twiddles(d->n, d->tw, dbl, p->st);
+        const bool col_dft = p->col_dft && d == &p->d2;
+        if (d->big || col_dft) {
+            FRES_TRY(dalloc(p, &d->tw, cs * d->n));
+            launch_twiddles(d->n, d->tw, dbl, p->st);
+        }
         if (d->big) {
             FRES_TRY(dalloc(p, &d->twa, cs * d->fpa.ntw));
             launch_stage_twiddles(d->fpa, d->twa, dbl, p->st);
             FRES_TRY(dalloc(p, &d->twb, cs * d->fpb.ntw));
             launch_stage_twiddles(d->fpb, d->twb, dbl, p->st);
-        } else {
+        } else if (!col_dft) {   // a direct column DFT needs none (gradients make them, adjoint_grid)
             FRES_TRY(dalloc(p, &d->stw, cs * d->fp.ntw));
             launch_stage_twiddles(d->fp, d->stw, dbl, p->st);
         }
@@ -1611,8 +1612,8 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
         FRES_TRY(dalloc(p, &p->ax, cs * p->n1 * p->B));
         FRES_TRY(dalloc(p, &p->ay, cs * p->n2 * p->B));
         // per problem: the chirp depends on lambda z
-        double* d_lz = nullptr;
-        FRES_TRY(dalloc(p, (void**)&d_lz, sizeof(double) * p->B));
+        // (their lambda z in the grid's first bytes until then: cleared below)
+        double* d_lz = (double*)p->grid;
         FRES_CK(cudaMemcpyAsync(d_lz, p->lzs.data(), sizeof(double) * p->B, cudaMemcpyHostToDevice, p->st));
         launch_t1_tables(p->B, d_lz, p->n1, p->nf1, p->opts.grid_h, p->opts.grid_x0, w, p->ks.beta, 1,
                          p->cps[0].sh1, p->ax, dbl, p->gq_t, p->gq_w, p->gq_n, p->st);
@@ -1668,6 +1669,8 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
         FRES_CK(cudaMemsetAsync(p->twork, 0, 2 * sizeof(int), p->st));
         p->ip.inv_tmax = 1.0 / tmax;
     }
+    // strip spreading adds into a zero grid; the row pass leaves it zero
+    if (p->strips) FRES_CK(cudaMemsetAsync(p->grid, 0, cs * (size_t)p->nf1 * p->nf2 * p->B, p->st));
     FRES_CK(cudaGetLastError());
     FRES_CK(cudaStreamSynchronize(p->st));
     return read_status(p);
@@ -1689,10 +1692,13 @@ namespace {
 template <typename T>
 fresnel_status adjoint_grid(Plan* p, const void* d_gamma) {
     const size_t cs = p->csize();
-    if (!p->adj_in) {
-        FRES_TRY(dalloc(p, &p->adj_in, cs * (size_t)p->n1 * p->n2 * p->B));
-        FRES_TRY(dalloc(p, &p->adj_rows, cs * (size_t)p->n2 * p->nf1 * p->B));
-        FRES_TRY(dalloc(p, (void**)&p->contrib, sizeof(double) * p->N));
+    // each on its own: a call that ran out of the memory cap may come again
+    if (!p->adj_in) FRES_TRY(dalloc(p, &p->adj_in, cs * (size_t)p->n1 * p->n2 * p->B));
+    if (!p->adj_rows) FRES_TRY(dalloc(p, &p->adj_rows, cs * (size_t)p->n2 * p->nf1 * p->B));
+    if (!p->contrib) FRES_TRY(dalloc(p, (void**)&p->contrib, sizeof(double) * p->N));
+    if (!p->d2.stw) {
+        FRES_TRY(dalloc(p, &p->d2.stw, cs * p->d2.fp.ntw));
+        launch_stage_twiddles(p->d2.fp, p->d2.stw, sizeof(T) == 8, p->st);
     }
     launch_adj_prologue<T>(d_gamma, p->ax, p->ay, p->adj_in, p->n1, p->n2, p->B,
                            p->output == FRESNEL_OCCULTER, p->st);

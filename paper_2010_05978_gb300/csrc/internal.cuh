@@ -153,6 +153,7 @@ struct ChirpParams {
     double kq;             // pi / lz
     double a1, a2, a0;     // phase = kq |x|^2 - a1 x - a2 y + a0 (pre-phase)
     int type3;
+    int row_base;          // added to a record's s2: problem * nf2 for strip-sorted plans, else 0
     // type 1: g = frac(x * u1) * nf1
     double u1, u2;
     // type 3: g = (x - C1) * inv_h1 + ng1 / 2
@@ -166,7 +167,6 @@ struct ChirpParams {
     // the wrap); the output tables undo it with exp(+2 pi i k sh / nf).
     int sh1, sh2;
     double screen_k;       // 2 pi / lambda of the problem (source screens)
-    int row_base;          // added to a record's s2: problem * nf2 for strip-sorted plans, else 0
 };
 
 // Piecewise-polynomial form of the spreading kernel: the value at
