@@ -262,37 +262,46 @@ k_interp_coop(const double* __restrict__ targets, long long M, const float2* __r
         }
         s_s[warp][lane] = make_int2(s1, s2);
         __syncwarp();
-        float gr = 0.0f, gi = 0.0f;
-#pragma unroll 1
-        for (int g = 0; g < 32 / TG; ++g) {
+        // LP steps, TG targets each; a lane's partial sum of every step stays in
+        // registers, and one transposing reduction over the LP lanes hands lane a
+        // the sum of step a: 2 LP shuffles per 32 targets instead of a reduction
+        // per step
+        float pr[LP], pi[LP];
+#pragma unroll
+        for (int g = 0; g < LP; ++g) {
             const int j = g * TG + sub;
             const int2 sj = s_s[warp][j];
             float rr = 0.0f, ri = 0.0f;
             if (a < W) {
-                const float kxa = s_kx[warp][j][a];
                 const float2* col = F + (long long)sj.y * ip.nfft1 + sj.x + a;
 #pragma unroll
                 for (int b = 0; b < W; ++b) {
                     const float2 v = __ldg(col + (long long)b * ip.nfft1);
-                    const float wgt = s_ky[warp][j][b] * kxa;
-                    rr = fmaf(wgt, v.x, rr);
-                    ri = fmaf(wgt, v.y, ri);
+                    const float kyb = s_ky[warp][j][b];
+                    rr = fmaf(kyb, v.x, rr);
+                    ri = fmaf(kyb, v.y, ri);
                 }
+                const float kxa = s_kx[warp][j][a];
+                rr *= kxa;
+                ri *= kxa;
             }
+            pr[g] = rr;
+            pi[g] = ri;
+        }
 #pragma unroll
-            for (int o = LP / 2; o > 0; o >>= 1) {
-                rr += __shfl_xor_sync(0xffffffffu, rr, o);
-                ri += __shfl_xor_sync(0xffffffffu, ri, o);
-            }
-            // lanes g TG .. g TG + TG - 1 own this step's targets: sum from lane (l - g TG) LP
-            const int src = ((lane - g * TG) * LP) & 31;
-            const float vr = __shfl_sync(0xffffffffu, rr, src);
-            const float vi = __shfl_sync(0xffffffffu, ri, src);
-            if (lane >= g * TG && lane < (g + 1) * TG) {
-                gr = vr;
-                gi = vi;
+        for (int o = LP / 2; o > 0; o >>= 1) {
+            const bool up = a & o;
+#pragma unroll
+            for (int i = 0; i < o; ++i) {
+                const float sr = up ? pr[i] : pr[i + o], si = up ? pi[i] : pi[i + o];
+                pr[i] = (up ? pr[i + o] : pr[i]) + __shfl_xor_sync(0xffffffffu, sr, o);
+                pi[i] = (up ? pi[i + o] : pi[i]) + __shfl_xor_sync(0xffffffffu, si, o);
             }
         }
+        // lane sub LP + a holds target a TG + sub
+        const int src = (lane % TG) * LP + lane / TG;
+        const float gr = __shfl_sync(0xffffffffu, pr[0], src);
+        const float gi = __shfl_sync(0xffffffffu, pi[0], src);
         __syncwarp();   // the next 32 targets overwrite the shared tables
         if (on) {
             const float dec = kernel_ft_cheb<float>(targ1, s_a, ncheb, inv_tmax) *
