@@ -208,10 +208,13 @@ typedef struct {
     const double* screen_opd;
     int screen_n1, screen_n2;
     double screen_box[4];
-    /* Bound on the one device-side wait of the spreading stage: the chunks
-     * of a tile that holds more records than one work item takes wait, before
-     * adding into the tile, for the flag with which the tile's first chunk
-     * reports having cleared it.  Polls per wait (~256 ns apart) before the
+    /* Bound on the one device-side wait of the spreading stage by tiles: the
+     * chunks of a tile that holds more records than one work item takes wait,
+     * before adding into the tile, for the flag with which the tile's first
+     * chunk reports having cleared it.  0 (default): plans spread by column
+     * strips, where nothing waits (by tiles, with the built-in bound, only
+     * where a memory cap leaves no room for the strip sort); any other value
+     * selects the tiles.  Polls per wait (~256 ns apart) before the
      * wait gives up, skips its addition and flags FRESNEL_ERR_TIMEOUT (read by
      * fresnel_check or a synchronous evaluation): 0 = the built-in 2^22
      * (about a second), > 0 = that many, < 0 = none at all (every such wait
