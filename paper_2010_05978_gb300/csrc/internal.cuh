@@ -329,6 +329,36 @@ struct ScanLayout {
 };
 constexpr int kMaxTileRows = 256;   // nf2 <= 8192
 
+// Programmatic dependent launch: a kernel launched with launch_after may be
+// scheduled while the kernel before it in the stream is still finishing.  It
+// first calls kernel_begin() in every thread of every block, before any memory
+// access or exit: that waits until the earlier kernel has completed and its
+// writes are visible, and only then lets the next kernel be scheduled, so at
+// most one kernel waits ahead and everything behaves as in stream order.  An
+// evaluation is three to seven kernels of 5 to 60 us; the gaps between them
+// cost 1 to 2 us each (us per call: disc 51 -> 42, star grid 87 -> 79, scattered
+// 161 -> 155, sweep 144 -> 138, kite 33.0 -> 31.1).  The strip spreading is
+// launched plainly: its blocks take very different times, and placed early, by
+// the room that the earlier kernel leaves, they load the SMs unevenly (kite 34.3,
+// star grid 80.6).
+__device__ __forceinline__ void kernel_begin() {
+    asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+void launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);   // errors: cudaGetLastError, as for <<<>>>
+}
+
 // ------------------------------------------------------------------ launchers
 // k_nodes.cu
 void launch_gauss_legendre(int n, double* t01, double* w01, cudaStream_t st);

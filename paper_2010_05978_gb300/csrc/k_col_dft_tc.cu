@@ -212,6 +212,7 @@ __global__ void __launch_bounds__(kTcThreads)
 k_col_dft_tc(ColPassArgs a, int n, unsigned nmask, unsigned* __restrict__ status) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     TcSmem& sm = *reinterpret_cast<TcSmem*>(smem_raw);
+    kernel_begin();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int b = blockIdx.z, c0 = blockIdx.x * kTcM;
     const int len = a.out_len;
@@ -367,7 +368,7 @@ void launch_col_dft_tc(const ColPassArgs& a, int n, unsigned* status, cudaStream
     const dim3 grid((a.ncols + kTcM - 1) / kTcM, (nchunks + kTcChunksPerCta - 1) / kTcChunksPerCta,
                     a.batch > 1 ? a.batch : 1);
     const unsigned nmask = (n & (n - 1)) == 0 ? (unsigned)(n - 1) : 0u;
-    k_col_dft_tc<<<grid, kTcThreads, smem, st>>>(a, n, nmask, status);
+    launch_after(k_col_dft_tc, grid, kTcThreads, smem, st, a, n, nmask, status);
 }
 
 }  // namespace fres

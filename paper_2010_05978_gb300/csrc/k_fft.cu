@@ -424,6 +424,7 @@ k_fft_rows(FftPlan fp, RowPassArgs a, int lines, int tr) {
     using C = cx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* S = (C*)smem_raw;
+    kernel_begin();
     const int n = fp.n;
     const C* tw = (const C*)a.twiddle;
     const T* dcol = (const T*)a.deconv_col;
@@ -469,6 +470,7 @@ k_fft_cols(FftPlan fp, ColPassArgs a, int ls) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ unsigned s_live[kMaxTileRows / 32];
     C* S = (C*)smem_raw;
+    kernel_begin();
     const int n = fp.n;
     const C* tw = (const C*)a.twiddle;
     const int ncol = 1 << ls, ngroups = (a.ncols + ncol - 1) >> ls;
@@ -672,8 +674,9 @@ void launch_fft_rows(const FftPlan& fp, const RowPassArgs& a, cudaStream_t st) {
     const int threads = (lines * tr + 31) / 32 * 32;
     const size_t smem = fft_smem<T>((size_t)lines * padded_len(fp.n) * sizeof(cx_t<T>));
     const int blocks = std::max(1, (nwork + lines - 1) / lines);
-    cudaFuncSetAttribute(k_fft_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_fft_rows<T><<<blocks, threads, smem, st>>>(fp, a, lines, tr);
+    if (smem > 48 * 1024)   // below, none is needed
+        cudaFuncSetAttribute(k_fft_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    launch_after(k_fft_rows<T>, blocks, threads, smem, st, fp, a, lines, tr);
 }
 
 template <typename T, int MODE>
@@ -691,9 +694,10 @@ void launch_cols_mode(const FftPlan& fp, const ColPassArgs& a, cudaStream_t st) 
     const int threads = ((fp.threads << ls) + 31) / 32 * 32;
     const size_t smem = fft_smem<T>(line << ls);
     const int blocks = (int)std::max(1LL, items(ls));
-    cudaFuncSetAttribute(k_fft_cols<T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    k_fft_cols<T, MODE><<<blocks, threads, smem, st>>>(fp, a, ls);
+    if (smem > 48 * 1024)
+        cudaFuncSetAttribute(k_fft_cols<T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem);
+    launch_after(k_fft_cols<T, MODE>, blocks, threads, smem, st, fp, a, ls);
 }
 
 // FP32 column passes of square type-3 grids, start (two buffers, radix-16/8/4/

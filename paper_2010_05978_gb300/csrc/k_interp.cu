@@ -224,6 +224,7 @@ k_interp_coop(const double* __restrict__ targets, long long M, const float2* __r
     __shared__ __align__(16) float s_kx[8][32][LP];
     __shared__ __align__(16) float s_ky[8][32][LP];
     __shared__ int2 s_s[8][32];
+    kernel_begin();
     for (int i = threadIdx.x; i < ncheb; i += blockDim.x) s_a[i] = (float)cheb[i];
     __syncthreads();
     const float inv_tmax = (float)ip.inv_tmax;
@@ -656,8 +657,8 @@ void launch_interp_w(const double* targets, long long M, const cx_t<T>* F, const
             const int cb = nblk(M, 256, 152 * 16);
 #define FRES_COOP_CASE(WW)                                                                     \
     case WW:                                                                                   \
-        k_interp_coop<WW><<<cb, 256, 0, st>>>(targets, M, F, ip, cheb, ncheb, (float2*)out,     \
-                                              status, ks.horner, beta);                        \
+        launch_after(k_interp_coop<WW>, cb, 256, 0, st, targets, M, F, ip, cheb, ncheb,        \
+                     (float2*)out, status, ks.horner, beta);                                   \
         return;
             switch (ks.w) {
                 FRES_COOP_CASE(2) FRES_COOP_CASE(3) FRES_COOP_CASE(4) FRES_COOP_CASE(5)

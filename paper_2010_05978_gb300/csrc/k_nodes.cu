@@ -596,6 +596,7 @@ __global__ void __launch_bounds__(kNodeThreads)
 k_nodes(FamTable ft, NodeRec<T>* rec, int* counts, StripSort ss, double* dx, double* dy,
         double* dw, unsigned* status) {
     __shared__ __align__(16) FamSmem sm;
+    kernel_begin();
     load_family(ft, sm);
     const FamilyDev& f = sm.f;
     const long long j = (long long)(blockIdx.x - sm.b0) * blockDim.x + threadIdx.x;
@@ -639,6 +640,7 @@ k_nodes(FamTable ft, NodeRec<T>* rec, int* counts, StripSort ss, double* dx, dou
 __global__ void __launch_bounds__(256) k_strip_starts(StripSort ss) {
     __shared__ int s_tot[8];
     __shared__ int s_base;
+    kernel_begin();
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int k0 = blockIdx.x * 1024 + 4 * t;   // nkeys is a multiple of 128
     int4 c = make_int4(0, 0, 0, 0);
@@ -678,6 +680,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_scatter_strips(long long n, const NodeRec<T>* __restrict__ rec, StripSort ss,
                  NodeRec<T>* __restrict__ sorted, unsigned* __restrict__ status) {
+    kernel_begin();
     const long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (j == 0) *ss.cursor = 0;   // the starts are done: ready for the next evaluation
     if (j >= n) return;
@@ -1162,7 +1165,8 @@ template <typename T>
 void launch_nodes_strips(const FamTable& ft, int nblocks, NodeRec<T>* rec, const StripSort& ss,
                          double* dx, double* dy, double* dw, unsigned* status, cudaStream_t st) {
     if (nblocks <= 0) return;
-    k_nodes<T, true><<<nblocks, kNodeThreads, 0, st>>>(ft, rec, nullptr, ss, dx, dy, dw, status);
+    launch_after(k_nodes<T, true>, nblocks, kNodeThreads, 0, st, ft, rec, nullptr, ss, dx, dy, dw,
+                 status);
 }
 template void launch_nodes_strips<float>(const FamTable&, int, NodeRec<float>*, const StripSort&,
                                          double*, double*, double*, unsigned*, cudaStream_t);
@@ -1170,13 +1174,13 @@ template void launch_nodes_strips<double>(const FamTable&, int, NodeRec<double>*
                                           double*, double*, double*, unsigned*, cudaStream_t);
 
 void launch_strip_starts(const StripSort& ss, cudaStream_t st) {
-    if (ss.nkeys > 0) k_strip_starts<<<nblk(ss.nkeys, 1024), 256, 0, st>>>(ss);
+    if (ss.nkeys > 0) launch_after(k_strip_starts, nblk(ss.nkeys, 1024), 256, 0, st, ss);
 }
 
 template <typename T>
 void launch_scatter_strips(long long n, const NodeRec<T>* rec, const StripSort& ss,
                            NodeRec<T>* sorted, unsigned* status, cudaStream_t st) {
-    if (n > 0) k_scatter_strips<T><<<nblk(n, 256), 256, 0, st>>>(n, rec, ss, sorted, status);
+    if (n > 0) launch_after(k_scatter_strips<T>, nblk(n, 256), 256, 0, st, n, rec, ss, sorted, status);
 }
 template void launch_scatter_strips<float>(long long, const NodeRec<float>*, const StripSort&,
                                            NodeRec<float>*, unsigned*, cudaStream_t);

@@ -62,6 +62,7 @@ k_spread_strips_f32(const NodeRec<float>* __restrict__ sorted, long long n, int 
     // the row reads free of bank conflicts
     __shared__ __align__(16) float s_kx[kStripWarps][32][M::COLS + 4];
     __shared__ __align__(16) float2 s_ck[kStripWarps][32][M::ROWS + 2];
+    kernel_begin();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long beg = ((long long)blockIdx.x * kStripWarps + warp) * range;
     if (beg >= n) return;   // no block-wide barrier follows
@@ -247,6 +248,7 @@ k_spread_strips_f64(const NodeRec<double>* __restrict__ sorted, long long n, int
     constexpr int NP = (W * W + 31) / 32;      // support cells per lane
     extern __shared__ __align__(16) unsigned char smem_raw[];
     StripSmemD<W>& sm = *reinterpret_cast<StripSmemD<W>*>(smem_raw);
+    kernel_begin();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long beg = ((long long)blockIdx.x * kStripWarps + warp) * range;
     if (beg >= n) return;   // no block-wide barrier follows
