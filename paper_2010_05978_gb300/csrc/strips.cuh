@@ -33,7 +33,7 @@
 // FP64 (k_spread_strips_f64): the FP64 pipe (1/58 of the FP32 rate) bounds
 // it, so no multiply-add goes to padding: lanes walk the w x w support
 // (ceil(w^2 / 32) steps) on a private 16-row window in shared memory.  Star,
-// w = 13: 1647 -> 703 us; w = 10: 1014 -> 424 us.
+// w = 13: 1647 -> 627 us; w = 10: 1014 -> 365 us.
 #pragma once
 #include "spread.cuh"
 
