@@ -91,6 +91,7 @@ struct Plan {
     // records sorted by strips and spread by k_spread_strips_* (strips.cuh);
     // else by tiles and k_spread / k_spread_det (see build_plan)
     bool strips = false;
+    bool strip_merge = false;     // a problem's sum may lie in a few cells
     StripSort ss{};
     KernelShape ks{};
     double sigma = 2.0;
@@ -684,7 +685,7 @@ fresnel_status eval_impl(Plan* p, const double* d_targets, long long M, void* d_
                              p->nf1, p->nf2, p->ntx, p->ntiles, p->ks, p->st);
         p->launches += p->max_split > 0 ? 3 : 2;
     } else if (p->strips) {
-        launch_spread_strips<T>((const NodeRec<T>*)p->sorted, p->N, p->ss.nkeys,
+        launch_spread_strips<T>((const NodeRec<T>*)p->sorted, p->N, p->chunk_cap, p->strip_merge,
                                 (cx_t<T>*)p->grid, p->nf1, p->nf2, p->ks, p->st);
         p->launches += 1;
     } else {
@@ -1442,8 +1443,29 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
     std::vector<int> tile_live(tt, -1), row_live(prune ? (size_t)p->B * p->nty : 0, 0);
     p->live_rows_total = 0;
     std::vector<int> rows;   // the row pass's work list (pruned plans)
+    // Strip spreading sums a block's rows before it adds them to the grid where
+    // much of a problem's sum may lie in a few cells (strips.cuh): problems of
+    // at most 16 live tiles or of 4096 records per live tile, starshades,
+    // explicit nodes (any weights) and peaked screens.  Elsewhere a node's
+    // weight is its share of the area, so a cell holds no more of the sum than
+    // of the aperture, however many nodes meet in it (the spokes of the
+    // dilation rule), and the merge would only cost its code's fetch and wide
+    // blocks (us per call, without and with it: disc 42 / 50, kite 31 / 37,
+    // star 86 / 88)
+    for (const FamilyDev& f : p->fams)
+        p->strip_merge |= f.kind == FRESNEL_FAMILY_PETALS || f.kind == FRESNEL_FAMILY_NODES;
+    if (p->opts.screen_n1 > 0 && p->opts.screen_amp) {
+        double most = 0.0, sum = 0.0;
+        const long long ns = (long long)p->opts.screen_n1 * p->opts.screen_n2;
+        for (long long i = 0; i < ns; ++i) {
+            most = std::max(most, std::fabs(p->opts.screen_amp[i]));
+            sum += std::fabs(p->opts.screen_amp[i]);
+        }
+        p->strip_merge |= !(most * ns <= 8.0 * sum);
+    }
     for (int b = 0; b < p->B; ++b) {
         long long nrec = 0, nsc = 0, nsplit = 0, nlive = 0;
+        const long long live0 = n_live;
         std::vector<char> live(p->nty, prune ? 0 : 1);
         for (int i = 0; i < p->ntiles; ++i)
             if (hc[(size_t)b * p->ntiles + i] > 0) {
@@ -1468,6 +1490,7 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
                 ++nsplit;
             }
         }
+        p->strip_merge |= n_live - live0 <= 16 || nrec >= 4096 * (n_live - live0);
         if (sc_off[b] + nsc + (long long)p->B * p->ntiles >= (1LL << 31) ||
             rec_off[b] + nrec >= (1LL << 31))
             return fres_fail(FRESNEL_ERR_UNSUPPORTED, "more than 2^31 records or chunks");

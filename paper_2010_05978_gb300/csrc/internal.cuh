@@ -420,10 +420,11 @@ void launch_spread(const NodeRec<T>* sorted, const Chunk* chunks, const int* n_m
                    int max_chunks, int* ready, int max_split, long long max_spin,
                    cx_t<T>* grid, int* work, unsigned* status, int nf1, int nf2, int ntx,
                    int ntiles, const KernelShape& ks, int nblocks, cudaStream_t st);
-// Strip-sorted records (strips.cuh): adds n records, sorted under nkeys keys,
-// into the grid, which must be zero; problems' grids are stacked by rows (record s2 = problem * nf2 + row).
+// Strip-sorted records (strips.cuh): adds n records into the grid, which must
+// be zero (merge: blocks of cap records add what they share once); problems'
+// grids are stacked by rows (record s2 = problem * nf2 + row).
 template <typename T>
-void launch_spread_strips(const NodeRec<T>* sorted, long long n, long long nkeys, cx_t<T>* grid,
+void launch_spread_strips(const NodeRec<T>* sorted, long long n, int cap, bool merge, cx_t<T>* grid,
                           int nf1, int nf2, const KernelShape& ks, cudaStream_t st);
 // Deterministic mode (fresnel_opts.deterministic): the same grid from exact
 // fixed-point sums, bit for bit whatever the records' order within a tile

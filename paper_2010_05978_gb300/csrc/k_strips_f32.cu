@@ -2,8 +2,8 @@
 #include "strips.cuh"
 namespace fres {
 template <>
-void launch_spread_strips<float>(const NodeRec<float>* sorted, long long n, long long nkeys, float2* grid,
+void launch_spread_strips<float>(const NodeRec<float>* sorted, long long n, int cap, bool merge, float2* grid,
                               int nf1, int nf2, const KernelShape& ks, cudaStream_t st) {
-    launch_strips_impl<float>(sorted, n, nkeys, grid, nf1, nf2, ks, st);
+    launch_strips_impl<float>(sorted, n, cap, merge, grid, nf1, nf2, ks, st);
 }
 }  // namespace fres

@@ -2,8 +2,8 @@
 #include "strips.cuh"
 namespace fres {
 template <>
-void launch_spread_strips<double>(const NodeRec<double>* sorted, long long n, long long nkeys, double2* grid,
+void launch_spread_strips<double>(const NodeRec<double>* sorted, long long n, int cap, bool merge, double2* grid,
                               int nf1, int nf2, const KernelShape& ks, cudaStream_t st) {
-    launch_strips_impl<double>(sorted, n, nkeys, grid, nf1, nf2, ks, st);
+    launch_strips_impl<double>(sorted, n, cap, merge, grid, nf1, nf2, ks, st);
 }
 }  // namespace fres

@@ -21,6 +21,18 @@
 // when the sweep moves.  The grid must be zero on entry: the row pass of the
 // FFT zeroes the nonzero cells that it reads.
 //
+// Rounding.  An addition to the grid rounds the whole sum of a cell, so where
+// much of a problem's sum lies in a few cells (a starshade on a coarse pupil
+// grid) the additions per cell decide the error.  Plans with such a problem
+// (see build_plan) run with MERGE: a block takes the tile kernel's chunk of
+// records (512 in FP32, 256 in FP64, more in large plans), its warps
+// neighbouring ranges of it, and the rows that the warps hold at the end are
+// summed in shared memory before they are added: a cell gets one addition per
+// block, strip and row sweep, about as many as the tile kernel made, whatever
+// the density.  FP32 adds in two levels besides, a batch's sums and the
+// range's: runs of 128 additions to one cell would round 10 to 25 % more than
+// the tile kernel's interleaved warps.
+//
 // FP32 (k_spread_strips_f32): accumulators in registers, a lane owning 4
 // columns of one row (w <= 8: 16 x 8 cells on 32 lanes; wider kernels own
 // more rows), so a record costs a 16-byte and an 8-byte shared load and 8
@@ -28,18 +40,72 @@
 // less than the tile kernel's read-modify-writes and duplicated records (1.5
 // per node at w = 8).  Bound by the shared-memory return path (6 words per
 // lane and record; L1 89 % busy at 4.3M records) and, where runs are short,
-// by issue.  Star at F = 100, 524,288 records: 61 -> 25 us; Koch snowflake,
-// 4.27M: 379 -> 127 us; F = 1000, 10.5M: 1.12 -> 0.52 ms.
+// by issue.  Cold L2, start (tiles) and now: star at F = 100, 524,288 records,
+// 65.5 -> 28.7 us; Koch snowflake, 4.27M, 379 -> 141 us; starshade sweep, 978k on 64
+// x 28 keys, 71.7 -> 32.8 us (MERGE; 34.8 without).
 // FP64 (k_spread_strips_f64): the FP64 pipe (1/58 of the FP32 rate) bounds
 // it, so no multiply-add goes to padding: lanes walk the w x w support
 // (ceil(w^2 / 32) steps) on a private 16-row window in shared memory.  Star,
-// w = 13: 1647 -> 627 us; w = 10: 1014 -> 365 us.
+// w = 13: 1649 -> 637 us; w = 10: 1016 -> 389 us.
 #pragma once
+#include <algorithm>
+
 #include "spread.cuh"
 
 namespace fres {
 
-constexpr int kStripWarps = 4;
+// Most warps of a block; MERGE: by registers (FP32: a lane holds one row up to
+// w = 8, then two, then four) and shared memory (FP64: 19 KB per warp at w = 16).
+template <typename T, int W, bool MERGE>
+constexpr int strip_warps() {
+    return !MERGE ? 4 : (sizeof(T) == 8 ? 12 : (W <= 8 ? 32 : (W == 9 ? 16 : 8)));
+}
+
+// The rows that the block's warps hold open at the end, added to the grid:
+// open = (strip, first row) of the calling warp (strip -1: none), whose cell
+// (y, x) is win(the warp's Smem, y, x), for open.y <= y < open.y + W.
+// Warps that hold the same strip of one tile row (neighbours: records are
+// sorted) are summed first, each adding its share of the rows.  V: the sum of
+// STEP neighbouring cells; add takes the first one's place in the (periodic,
+// stacked) grids and the sum.
+template <typename V, int W, int COLS, int STEP, class Smem, class Win, class Add>
+__device__ __forceinline__ void add_open_rows(Smem* sm, int2 open, int nf1, int nf2, Win win, Add add) {
+    __shared__ int2 s_open[32];
+    constexpr int QC = COLS / STEP;
+    const int warps = blockDim.x >> 5, lane = threadIdx.x & 31, me = threadIdx.x >> 5;
+    if (lane == 0) s_open[me] = open;
+    __syncthreads();
+    // this warp's neighbours v .. e - 1 of the same strip, first rows ascending
+    const int2 o = lane < warps ? s_open[lane] : make_int2(-1, 0);
+    const int pa = __shfl_up_sync(0xffffffffu, o.x, 1), pb = __shfl_up_sync(0xffffffffu, o.y, 1);
+    const unsigned first = __ballot_sync(
+        0xffffffffu, lane == 0 || lane >= warps || o.x != pa || (o.y >> 5) != (pb >> 5) || o.y < pb);
+    const int v = 31 - __clz(first & (0xffffffffu >> (31 - me)));
+    const unsigned next = me < 31 ? first >> (me + 1) : 0u;
+    const int e = next ? me + __ffs(next) : warps;
+    if (open.x >= 0) {
+        const int y0 = s_open[v].y, yend = (y0 / nf2 + 1) * nf2;
+        for (int t = (me - v) * 32 + lane; t < (s_open[e - 1].y - y0 + W) * QC; t += (e - v) * 32) {
+            const int y = y0 + t / QC, x = t % QC * STEP;
+            V s{};
+            for (int u = v; u < e; ++u) {
+                const int d = y - s_open[u].y;
+                if (d >= 0 && d < W) {
+                    const V c = win(sm[u], y, x);
+                    s.x += c.x;
+                    s.y += c.y;
+                    if constexpr (STEP == 2) {
+                        s.z += c.z;
+                        s.w += c.w;
+                    }
+                }
+            }
+            int gx = open.x * 8 + x;
+            if (gx >= nf1) gx -= nf1;
+            add(gx, y >= yend ? y - nf2 : y, s);
+        }
+    }
+}
 
 // ------------------------------------------------------------------ FP32
 template <int W>
@@ -52,28 +118,35 @@ struct StripMap {
     static constexpr int NQ = (W + 3 + 3) / 4;           // quads of a kernel row shifted by 0..3
 };
 
-// DENSE: sums in two levels, a batch's and the range's (see strip_dense).
-template <int W, bool DENSE>
-__global__ void __launch_bounds__(kStripWarps * 32)
+// 16-byte rows whose strides (20 or 36 words) keep the staging stores and
+// the row reads free of bank conflicts.  At the end a warp's open rows take
+// the place of kx: row y in slot y mod ROWS
+template <int W>
+struct StripSmemF {
+    using M = StripMap<W>;
+    float kx[32][M::COLS + 4];
+    float2 ck[32][M::ROWS + 2];
+};
+
+template <int W, bool MERGE>
+__global__ void __launch_bounds__(strip_warps<float, W, MERGE>() * 32)
 k_spread_strips_f32(const NodeRec<float>* __restrict__ sorted, long long n, int range,
                     float2* __restrict__ grid, int nf1, int nf2, float beta, const HornerTab hz) {
     using M = StripMap<W>;
-    // 16-byte rows whose strides (20 or 36 words) keep the staging stores and
-    // the row reads free of bank conflicts
-    __shared__ __align__(16) float s_kx[kStripWarps][32][M::COLS + 4];
-    __shared__ __align__(16) float2 s_ck[kStripWarps][32][M::ROWS + 2];
+    static_assert(M::ROWS * M::COLS * sizeof(float2) <= sizeof(StripSmemF<W>::kx), "open rows");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    StripSmemF<W>* sm = reinterpret_cast<StripSmemF<W>*>(smem_raw);
     kernel_begin();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long beg = ((long long)blockIdx.x * kStripWarps + warp) * range;
-    if (beg >= n) return;   // no block-wide barrier follows
-    const long long end = beg + range < n ? beg + range : n;
-    float(*kx)[M::COLS + 4] = s_kx[warp];
-    float2(*ck)[M::ROWS + 2] = s_ck[warp];
+    const long long beg = ((long long)blockIdx.x * (blockDim.x >> 5) + warp) * range;
+    const long long end = beg + range < n ? beg + range : n;   // <= beg: no records
+    float(*kx)[M::COLS + 4] = sm[warp].kx;
+    float2(*ck)[M::ROWS + 2] = sm[warp].ck;
 #pragma unroll
     for (int b = W; b < M::ROWS; ++b) ck[lane][b] = make_float2(0.0f, 0.0f);
     const int cg = lane % M::COLG, rg = lane / M::COLG;
-    float2 acc[M::RPL][4];
-    float2 sum[DENSE ? M::RPL : 1][4];   // DENSE: the earlier batches'
+    float2 acc[M::RPL][4];           // this batch's sums
+    float2 sum[M::RPL][4];           // the earlier batches'
     int slot[M::RPL];                // this lane's rows relative to the open row
     const float2* ckp[M::RPL];       // their staged values (of record 0)
     const float4* kxp = reinterpret_cast<const float4*>(&kx[0][4 * cg]);
@@ -86,11 +159,16 @@ k_spread_strips_f32(const NodeRec<float>* __restrict__ sorted, long long n, int 
         slot[k] = 0;
         ckp[k] = &ck[0][0];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            acc[k][i] = make_float2(0.0f, 0.0f);
-            if constexpr (DENSE) sum[k][i] = make_float2(0.0f, 0.0f);
-        }
+        for (int i = 0; i < 4; ++i) acc[k][i] = sum[k][i] = make_float2(0.0f, 0.0f);
     }
+    auto fold = [&](int k) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            sum[k][i].x += acc[k][i].x;
+            sum[k][i].y += acc[k][i].y;
+            acc[k][i] = make_float2(0.0f, 0.0f);
+        }
+    };
     // adds the rows less than d below the open one to the grid (a row's zero
     // cells too: they stay inside the grid, and testing costs more)
     auto flush = [&](int d) {
@@ -100,24 +178,17 @@ k_spread_strips_f32(const NodeRec<float>* __restrict__ sorted, long long n, int 
                 int y = cur_b + slot[k];
                 if (y >= yend) y -= nf2;
                 float2* dst = colp + (long long)y * nf1;
-                if constexpr (DENSE) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        acc[k][i].x += sum[k][i].x;
-                        acc[k][i].y += sum[k][i].y;
-                        sum[k][i] = make_float2(0.0f, 0.0f);
-                    }
-                }
+                fold(k);
                 asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst),
-                             "f"(acc[k][0].x), "f"(acc[k][0].y), "f"(acc[k][1].x),
-                             "f"(acc[k][1].y)
+                             "f"(sum[k][0].x), "f"(sum[k][0].y), "f"(sum[k][1].x),
+                             "f"(sum[k][1].y)
                              : "memory");
                 asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + 2),
-                             "f"(acc[k][2].x), "f"(acc[k][2].y), "f"(acc[k][3].x),
-                             "f"(acc[k][3].y)
+                             "f"(sum[k][2].x), "f"(sum[k][2].y), "f"(sum[k][3].x),
+                             "f"(sum[k][3].y)
                              : "memory");
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[k][i] = make_float2(0.0f, 0.0f);
+                for (int i = 0; i < 4; ++i) sum[k][i] = make_float2(0.0f, 0.0f);
             }
     };
     NodeRec<float> r{};
@@ -215,45 +286,63 @@ k_spread_strips_f32(const NodeRec<float>* __restrict__ sorted, long long n, int 
                 }
             }
         }
-        if constexpr (DENSE) {
 #pragma unroll
-            for (int k = 0; k < M::RPL; ++k)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    sum[k][i].x += acc[k][i].x;
-                    sum[k][i].y += acc[k][i].y;
-                    acc[k][i] = make_float2(0.0f, 0.0f);
-                }
-        }
+        for (int k = 0; k < M::RPL; ++k) fold(k);
         __syncwarp();   // the next batch overwrites the staged values
     }
-    if (cur_a >= 0) flush(M::ROWS);
+    if constexpr (!MERGE) {
+        if (cur_a >= 0) flush(M::ROWS);
+        return;
+    }
+    // what is still open, summed over the block's warps
+    float2* win = reinterpret_cast<float2*>(kx);
+#pragma unroll
+    for (int k = 0; k < M::RPL; ++k) {
+        fold(k);
+#pragma unroll
+        for (int i = 0; i < 4; i += 2)
+            *reinterpret_cast<float4*>(win + (rg + k * M::RSTEP) * M::COLS + 4 * cg + i) =
+                make_float4(sum[k][i].x, sum[k][i].y, sum[k][i + 1].x, sum[k][i + 1].y);
+    }
+    add_open_rows<float4, W, M::COLS, 2>(
+        sm, make_int2(cur_a, cur_b), nf1, nf2,
+        [](const StripSmemF<W>& w, int y, int x) {
+            return *reinterpret_cast<const float4*>(reinterpret_cast<const float2*>(w.kx) +
+                                                    (y & (M::ROWS - 1)) * M::COLS + x);
+        },
+        [&](int x, int y, float4 v) {
+            if (v.x == 0.0f && v.y == 0.0f && v.z == 0.0f && v.w == 0.0f) return;
+            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(
+                             grid + (long long)y * nf1 + x),
+                         "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+                         : "memory");
+        });
 }
 
 // ------------------------------------------------------------------ FP64
 template <int W>
 struct StripSmemD {
     static constexpr int COLS = W + 7;
-    double2 win[kStripWarps][16 * COLS];
-    double2 ck[kStripWarps][32][W | 1];
-    double kx[kStripWarps][32][W | 1];
+    double2 win[16 * COLS];
+    double2 ck[32][W | 1];
+    double kx[32][W | 1];
 };
 
-template <int W>
-__global__ void __launch_bounds__(kStripWarps * 32)
+template <int W, bool MERGE>
+__global__ void __launch_bounds__(strip_warps<double, W, MERGE>() * 32)
 k_spread_strips_f64(const NodeRec<double>* __restrict__ sorted, long long n, int range,
                     double2* __restrict__ grid, int nf1, int nf2, double beta,
                     const HornerTabD hz) {
     constexpr int COLS = StripSmemD<W>::COLS;
     constexpr int NP = (W * W + 31) / 32;      // support cells per lane
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    StripSmemD<W>& sm = *reinterpret_cast<StripSmemD<W>*>(smem_raw);
     kernel_begin();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long beg = ((long long)blockIdx.x * kStripWarps + warp) * range;
-    if (beg >= n) return;   // no block-wide barrier follows
-    const long long end = beg + range < n ? beg + range : n;
-    double2* win = sm.win[warp];
+    StripSmemD<W>* all = reinterpret_cast<StripSmemD<W>*>(smem_raw);
+    StripSmemD<W>& sm = all[warp];
+    const long long beg = ((long long)blockIdx.x * (blockDim.x >> 5) + warp) * range;
+    const long long end = beg + range < n ? beg + range : n;   // <= beg: no records
+    double2* win = sm.win;
     for (int e = lane; e < 16 * COLS; e += 32) win[e] = make_double2(0.0, 0.0);
     int ca[NP], cb[NP], off[NP];               // cell (a, b) of step k, its window offset
 #pragma unroll
@@ -294,11 +383,11 @@ k_spread_strips_f64(const NodeRec<double>* __restrict__ sorted, long long n, int
             double kv[W];
             kernel_values<double, W>(r.f1, beta, hz, kv);
 #pragma unroll
-            for (int i = 0; i < W; ++i) sm.kx[warp][lane][i] = kv[i];
+            for (int i = 0; i < W; ++i) sm.kx[lane][i] = kv[i];
             kernel_values<double, W>(r.f2, beta, hz, kv);
 #pragma unroll
             for (int i = 0; i < W; ++i)
-                sm.ck[warp][lane][i] = make_double2(r.cre * kv[i], r.cim * kv[i]);
+                sm.ck[lane][i] = make_double2(r.cre * kv[i], r.cim * kv[i]);
         }
         if (base + 32 + lane < end) r = sorted[base + 32 + lane];
         int pa = __shfl_up_sync(0xffffffffu, a, 1), pb = __shfl_up_sync(0xffffffffu, b, 1);
@@ -325,8 +414,8 @@ k_spread_strips_f64(const NodeRec<double>* __restrict__ sorted, long long n, int
 #pragma unroll
             for (int k = 0; k < NP; ++k)
                 if (cb[k] < W) {
-                    const double kv = sm.kx[warp][j][ca[k]];
-                    const double2 c = sm.ck[warp][j][cb[k]];
+                    const double kv = sm.kx[j][ca[k]];
+                    const double2 c = sm.ck[j][cb[k]];
                     double2* cell = win + off[k] + x0;
                     double2 o = *cell;
                     o.x += c.x * kv;
@@ -336,67 +425,77 @@ k_spread_strips_f64(const NodeRec<double>* __restrict__ sorted, long long n, int
             __syncwarp();
         }
     }
-    if (cur_a >= 0) flush(W);
-}
-
-// Where the keys hold many records each (a starshade on a few cells: 35; the
-// star at F = 100: 6) every warp adds to the same cells of the grid, and each
-// addition there rounds the whole sum: longer ranges, summed in two levels so
-// that they round no worse themselves.  With one level, repeats of the sweep's
-// eight-wavelength design differed by 2.7e-6 (32 records per warp), 1.3e-6
-// (128) and 1.2e-6 (256), against the tile kernel's 0.9e-6.
-// FP64 (one level) from 64 records per key on: 311,297 nodes, a third of them
-// on one point, 1.4e-13 from the exact sums at 64 records per warp, against the tile
-// kernel's 0.4e-13.
-inline bool strip_dense(long long n, long long nkeys, bool dbl) {
-    return n >= (dbl ? 64 : 16) * nkeys;
-}
-
-// Records per warp.  FP32: enough warps for every SM's resident set (152 x
-// 32), at least one batch and at most four: 128 consecutive additions to a
-// cell, as many as the tile kernel's warps make; eight batches where dense.
-// FP64 records cost far more than a flush, so the split that balances the SMs
-// wins: two batches per warp (w = 13: 703 us at 128 records, 627 at 32), one
-// below 16 warps per SM, dense or not (81,120 nodes of five starshades, w = 10:
-// 176 us at 256).
-inline int strip_range(long long n, bool dense, bool dbl) {
-    if (dbl && n < 152LL * 16 * 64) return 32;
-    if (dense) return 256;
-    if (dbl) return 64;
-    const long long r = (n / (152 * 32) + 31) / 32 * 32;
-    return (int)(r < 32 ? 32 : (r > 128 ? 128 : r));
-}
-
-template <typename T, int W>
-void launch_strips_w(const NodeRec<T>* sorted, long long n, long long nkeys, cx_t<T>* grid,
-                     int nf1, int nf2, const KernelShape& ks, cudaStream_t st) {
-    const bool dense = (W <= 9 || sizeof(T) == 8) && strip_dense(n, nkeys, sizeof(T) == 8);
-    const int range = strip_range(n, dense, sizeof(T) == 8);
-    const long long warps = (n + range - 1) / range;
-    const int blocks = (int)((warps + kStripWarps - 1) / kStripWarps);
-    if constexpr (sizeof(T) == 4) {
-        if (dense)
-            k_spread_strips_f32<W, (W <= 9)><<<blocks, kStripWarps * 32, 0, st>>>(
-                sorted, n, range, grid, nf1, nf2, ks.betaf, ks.horner);
-        else
-            k_spread_strips_f32<W, false><<<blocks, kStripWarps * 32, 0, st>>>(
-                sorted, n, range, grid, nf1, nf2, ks.betaf, ks.horner);
-    } else {
-        const size_t smem = sizeof(StripSmemD<W>);
-        cudaFuncSetAttribute(k_spread_strips_f64<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-        k_spread_strips_f64<W><<<blocks, kStripWarps * 32, smem, st>>>(
-            sorted, n, range, grid, nf1, nf2, ks.beta, ks.hornerd);
+    if constexpr (!MERGE) {
+        if (cur_a >= 0) flush(W);
+        return;
     }
+    add_open_rows<double2, W, COLS, 1>(
+        all, make_int2(cur_a, cur_b), nf1, nf2,
+        [](const StripSmemD<W>& w, int y, int x) { return w.win[(y & 15) * COLS + x]; },
+        [&](int x, int y, double2 v) {
+            if (v.x == 0.0 && v.y == 0.0) return;
+            double2* g = grid + (long long)y * nf1 + x;
+            atomicAdd(&g->x, v.x);
+            atomicAdd(&g->y, v.y);
+        });
+}
+
+// Records per warp and warps per block.  FP32: enough warps for every SM's
+// resident set (152 x 32), at least one batch and at most four.  FP64 records
+// cost far more than a flush, so the split that balances the SMs wins: two
+// batches per warp, one below 16 warps per SM.  MERGE: a block takes `cap`
+// records, the plan's chunk of the tile kernel, or up to twice as many where
+// that loads the fullest SM less (117,000 records: 800 instead of 2 x 512); in
+// large FP32 plans (cap above its base) eight warps, so that the last blocks
+// are short.
+inline void strip_shape(long long n, int cap, bool dbl, bool merge, int most, int* range, int* warps) {
+    const int base = dbl ? 256 : 512;
+    const int few = dbl ? 64 : 128;
+    long long r = dbl ? (n < 152LL * 16 * 64 ? 32 : 64) : (n / (152 * 32) + 31) / 32 * 32;
+    r = r < 32 ? 32 : (r > few ? few : r);
+    *warps = most;
+    *range = (int)r;
+    if (!merge) return;
+    while (base % r || base / r > most) r += 32;   // 32, 64 or 128
+    int w = !dbl && cap > base ? 8 : (int)(base / r);
+    long long load = -1;
+    for (int k = w; cap == base && k <= std::min(most, (int)(2 * base / r)); ++k) {
+        const long long per = k * r, l = ((n + per - 1) / per + 151) / 152 * per;
+        if (load < 0 || l < load) {
+            load = l;
+            w = k;
+        }
+    }
+    *warps = w;
+    *range = std::max((int)r, (cap / w + 31) / 32 * 32);
+}
+
+template <typename T, int W, bool MERGE>
+void launch_strips_w(const NodeRec<T>* sorted, long long n, int cap, cx_t<T>* grid, int nf1, int nf2,
+                     const KernelShape& ks, cudaStream_t st) {
+    int range, warps;
+    strip_shape(n, cap, sizeof(T) == 8, MERGE, strip_warps<T, W, MERGE>(), &range, &warps);
+    const long long per = (long long)range * warps;
+    auto launch = [&](auto kernel, size_t smem, auto beta, const auto& horner) {
+        if (smem > 48 * 1024)
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        kernel<<<(unsigned)((n + per - 1) / per), warps * 32, smem, st>>>(sorted, n, range, grid, nf1,
+                                                                          nf2, beta, horner);
+    };
+    if constexpr (sizeof(T) == 4)
+        launch(k_spread_strips_f32<W, MERGE>, warps * sizeof(StripSmemF<W>), ks.betaf, ks.horner);
+    else
+        launch(k_spread_strips_f64<W, MERGE>, warps * sizeof(StripSmemD<W>), ks.beta, ks.hornerd);
 }
 
 template <typename T>
-void launch_strips_impl(const NodeRec<T>* sorted, long long n, long long nkeys, cx_t<T>* grid,
+void launch_strips_impl(const NodeRec<T>* sorted, long long n, int cap, bool merge, cx_t<T>* grid,
                         int nf1, int nf2, const KernelShape& ks, cudaStream_t st) {
     if (n <= 0) return;
-#define FRES_STRIP_CASE(WW)                                          \
-    case WW:                                                         \
-        launch_strips_w<T, WW>(sorted, n, nkeys, grid, nf1, nf2, ks, st); \
+#define FRES_STRIP_CASE(WW)                                                                  \
+    case WW:                                                                                 \
+        if (merge) launch_strips_w<T, WW, true>(sorted, n, cap, grid, nf1, nf2, ks, st);     \
+        else launch_strips_w<T, WW, false>(sorted, n, cap, grid, nf1, nf2, ks, st);          \
         break;
     switch (ks.w) {
         FRES_STRIP_CASE(2) FRES_STRIP_CASE(3) FRES_STRIP_CASE(4) FRES_STRIP_CASE(5)
