@@ -1184,6 +1184,8 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
         ip.occulter = p->output == FRESNEL_OCCULTER;
     }
     // FFT lengths: one shared-memory pass, or the four-step split
+    bool petals = false;
+    for (const FamilyDev& f : p->fams) petals |= f.kind == FRESNEL_FAMILY_PETALS;
     for (FftDim* d : {&p->d1, &p->d2}) {
         d->n = d == &p->d1 ? p->nfft1 : p->nfft2;
         const bool forced = p->opts.fft_split_above > 0 && d->n > p->opts.fft_split_above;
@@ -1194,7 +1196,7 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
                                 p->opts.fft_split_above == 0 && p->opts.max_device_bytes == 0 &&
                                 d->n > kSplitColumnsAbove && fft_split(d->n, dbl, &d->fa, &d->fb);
         if (fft_supported(d->n, dbl) && !forced && !split_cols) {
-            d->fp = make_fft_plan(d->n, dbl);
+            d->fp = make_fft_plan(d->n, dbl, petals && p->tkind == FRESNEL_GRID);
         } else if (fft_split(d->n, dbl, &d->fa, &d->fb)) {
             d->big = true;
             d->fpa = make_fft_plan(d->fa, dbl);

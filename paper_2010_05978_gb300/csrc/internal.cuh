@@ -552,7 +552,7 @@ void launch_col_pfft_d(const ColPassArgs& a, int n, unsigned* status, cudaStream
 bool fft_supported(int n, int is_double);
 // Split of a length beyond one pass into fa * fb (both single-pass), or false.
 bool fft_split(int n, int is_double, int* fa, int* fb);
-FftPlan make_fft_plan(int n, int is_double);   // nstages < 0: no plan
+FftPlan make_fft_plan(int n, int is_double, bool plain = false);   // nstages < 0: no plan
 
 // k_interp.cu
 struct InterpParams {
