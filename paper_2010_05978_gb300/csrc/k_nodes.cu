@@ -110,7 +110,13 @@ __device__ __forceinline__ void legendre_pn(int n, double x, const double2* c, d
 #pragma unroll 4
     for (int j = 1; j < n; ++j) {
         // only the multiply-add is on the chain p0, p1 -> p2
-        const double2 k = kTable ? c[j] : make_double2((2.0 * j + 1.0) / (j + 1.0), j / (j + 1.0));
+        double2 k;
+        if (kTable) {
+            k = c[j];
+        } else {
+            const double inv = 1.0 / (j + 1.0);
+            k = make_double2((2.0 * j + 1.0) * inv, j * inv);
+        }
         const double p2 = fma(k.x * x, p1, -(k.y * p0));
         p0 = p1;
         p1 = p2;
@@ -138,16 +144,18 @@ __global__ void k_gauss_legendre(int n, double* t01, double* w01) {
     double x = (1.0 - (nn - 1.0) / (8.0 * nn * nn * nn)) * cos(kPi * (i + 0.75) / (nn + 0.5));
     if (2 * i + 1 == n) x = 0.0;   // odd n: the middle root
     double pn, pn1;
-    // Newton squares the error (times x/(1 - x^2), below n^2/5 at the end
-    // roots), so a step below 1e-11 leaves the root exact to rounding: two or
-    // three steps, each a chain of n dependent recurrences, instead of the
-    // four or five until two steps in a row had vanished
+    // Newton squares the error, times x/(1 - x^2): below n^2/5 at the end
+    // roots.  A step below 3e-9 / n therefore leaves 2e-18, a root exact to
+    // rounding (1e-11 alone left 1.5e-14 and end weights 5e-6 off at n =
+    // 31,000): two or three steps, each a chain of n dependent recurrences,
+    // instead of the four or five until two steps in a row had vanished
+    const double enough = fmin(1e-11, 3e-9 / nn);
     for (int it = 0; it < 100; ++it) {
         legendre_pn<kTable>(n, x, s_c, &pn, &pn1);
         const double dp = nn * (x * pn - pn1) / (x * x - 1.0);
         const double dx = pn / dp;
         x -= dx;
-        if (fabs(dx) < 1e-11) break;
+        if (fabs(dx) < enough) break;
     }
     legendre_pn<kTable>(n, x, s_c, &pn, &pn1);
     const double dp = nn * (x * pn - pn1) / (x * x - 1.0);
@@ -1129,7 +1137,11 @@ inline int nblk(long long n, int b) { return (int)((n + b - 1) / b); }
 void launch_gauss_legendre(int n, double* t01, double* w01, cudaStream_t st) {
     const size_t dyn = sizeof(double2) * (size_t)n;
     const int blocks = nblk((n + 1) / 2, 64);
-    if (dyn <= 48 * 1024) {
+    // the table up to n = 6143 (n = 5000: plan 11.9 ms without it, 2.5 with)
+    if (n < 6144) {
+        if (dyn > 48 * 1024)
+            cudaFuncSetAttribute(k_gauss_legendre<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)dyn);
         k_gauss_legendre<true><<<blocks, 64, dyn, st>>>(n, t01, w01);
     } else {
         k_gauss_legendre<false><<<blocks, 64, 0, st>>>(n, t01, w01);
