@@ -116,8 +116,8 @@ struct Plan {
     FftDim d1{}, d2{};            // FFT along x (rows) and y (columns)
     void* fscratch = nullptr;     // four-step intermediate
     std::vector<void*> allocs;
-    char* slab = nullptr;         // small allocations are carved from 1 MB slabs (in allocs)
-    size_t slab_left = 0;
+    char* slab = nullptr;         // small allocations are carved from slabs (in allocs)
+    size_t slab_left = 0, slab_size = 0;
     long long bytes = 0;
     void* rec = nullptr;
     void* sorted = nullptr;
@@ -206,24 +206,28 @@ fresnel_status dalloc(Plan* p, void** out, size_t bytes) {
     if (p->opts.max_device_bytes > 0 && p->bytes + (long long)bytes > p->opts.max_device_bytes)
         return fres_fail(FRESNEL_ERR_OOM, "plan would exceed max_device_bytes (" +
                                                std::to_string(p->opts.max_device_bytes) + ")");
-    // A plan holds a dozen small tables per family: carved from slabs they cost
-    // one cudaMalloc and cudaFree per megabyte (an eight-wavelength starshade
-    // plan: 240 -> 20 of each).  Under a memory cap every allocation is its own,
-    // so that the cap counts all that is held.
+    // A plan holds a dozen small tables per family: carved from slabs of 64 KB,
+    // doubling to 1 MB, they cost a few cudaMalloc and cudaFree in all (an
+    // eight-wavelength starshade plan: 240 -> 20 of each).  Whole slabs count as
+    // held.  Under a memory cap every allocation is its own, so that the cap
+    // counts all that is held.
     constexpr size_t kSlab = 1 << 20, kSmall = 64 << 10;
     const bool small = bytes <= kSmall && p->opts.max_device_bytes == 0;
     const size_t carve = (bytes + 255) & ~(size_t)255;
     if (!small || p->slab_left < carve) {
-        cudaError_t e = cudaMalloc(out, small ? kSlab : bytes);
+        if (small) p->slab_size = std::min(kSlab, std::max(kSmall, 2 * p->slab_size));
+        const size_t held = small ? p->slab_size : bytes;
+        cudaError_t e = cudaMalloc(out, held);
         if (e != cudaSuccess) {
             *out = nullptr;
             cudaGetLastError();
             return fres_fail(FRESNEL_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
         }
         p->allocs.push_back(*out);
+        p->bytes += (long long)held;
         if (small) {
             p->slab = (char*)*out;
-            p->slab_left = kSlab;
+            p->slab_left = held;
         }
     }
     if (small) {
@@ -231,7 +235,6 @@ fresnel_status dalloc(Plan* p, void** out, size_t bytes) {
         p->slab += carve;
         p->slab_left -= carve;
     }
-    p->bytes += (long long)bytes;
     return FRESNEL_OK;
 }
 

@@ -1,0 +1,43 @@
+"""Device memory of plans: what info() reports is what is held, small plans hold
+little, and plans that fit in the memory that is left are not refused."""
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+MB = 1 << 20
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2010_05978_gb300 import build
+    build.build()
+    torch.cuda.set_device(0)
+
+
+def _free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+@pytest.mark.parametrize("kind", ["grid", "scattered"])
+def test_held_memory_is_reported_and_small_plans_hold_little(kind):
+    from paper_2010_05978_gb300 import Plan
+    fam = W.fourier_family([1.0, 0.02, 0.01], 12, 8, 12)
+    where = {"grid": {"grid": W.grid_spec(24, 24, 0.05)}, "scattered": {"box": (-1, 1, -1, 1)}}[kind]
+    # FP64: FP32 scattered plans have a stream of their own, which takes device
+    # memory (0.6 MB) that is no allocation of the plan's
+    make = lambda **kw: Plan([fam], 0.5, 1.0, 1e-6, precision="fp64", **where, **kw)
+    make().close()
+    exact = make(max_device_bytes=1 << 40).info()["device_bytes"]   # every allocation its own
+    before = _free()
+    plans = [make() for _ in range(200)]
+    held, reported = before - _free(), sum(p.info()["device_bytes"] for p in plans)
+    # cudaMalloc takes memory from the device 2 MB at a time
+    assert held <= 1.05 * reported + 4 * MB
+    # at most as much again in the slabs as the tables in them, and one slab more
+    assert plans[0].info()["device_bytes"] <= 2 * exact + (64 << 10)
