@@ -114,6 +114,7 @@ struct Plan {
     InterpParams ip{};
     FftPlan fp1{}, fp2{};
     FftDim d1{}, d2{};            // FFT along x (rows) and y (columns)
+    bool split_cols = false;      // columns in four steps though one pass would do
     void* fscratch = nullptr;     // four-step intermediate
     std::vector<void*> allocs;
     char* slab = nullptr;         // small allocations are carved from slabs (in allocs)
@@ -1195,9 +1196,12 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
         // FP32 scattered plans (one problem, no gradients: nothing else needs
         // single passes) split long columns too: a single pass takes two
         // columns per block there, 16 of a sector's 32 bytes
+        // (when the scratch grid does not fit, the plan is built without:
+        // fresnel_plan_many)
         const bool split_cols = d == &p->d2 && !dbl && p->tkind == FRESNEL_SCATTERED &&
                                 p->opts.fft_split_above == 0 && p->opts.max_device_bytes == 0 &&
                                 d->n > kSplitColumnsAbove && fft_split(d->n, dbl, &d->fa, &d->fb);
+        p->split_cols |= split_cols && fft_supported(d->n, dbl);
         if (fft_supported(d->n, dbl) && !forced && !split_cols) {
             d->fp = make_fft_plan(d->n, dbl, petals && p->tkind == FRESNEL_GRID);
         } else if (fft_split(d->n, dbl, &d->fa, &d->fb)) {
@@ -1958,9 +1962,13 @@ fresnel_status fresnel_plan_many(const fresnel_problem* problems, int n_problems
     if (s != FRESNEL_OK) {
         std::string msg = g_last_error;
         cudaGetLastError();
+        const bool again = s == FRESNEL_ERR_OOM && p->split_cols;
         free_plan(p);
         g_last_error = msg;
-        return s;
+        if (!again) return s;
+        fresnel_opts o = *opts;   // without the columns' scratch grid
+        o.fft_split_above = INT_MAX;
+        return fresnel_plan_many(problems, n_problems, tol, &o, cuda_stream, out_plan);
     }
     *out_plan = reinterpret_cast<fresnel_plan_t>(p);
     return FRESNEL_OK;
@@ -2243,7 +2251,13 @@ fresnel_status plan_scattered_batch(const fresnel_problem* problems, int n, doub
         fresnel_status st = fresnel_plan_many(&problems[b], 1, tol, &so, stream, &h);
         if (st != FRESNEL_OK) {
             g_last_error = "problem " + std::to_string(b) + ": " + g_last_error;
-            return fail(st);
+            bool again = false;
+            for (const Plan* q : p->subs) again |= q->split_cols;
+            if (st != FRESNEL_ERR_OOM || !again) return fail(st);
+            fail(st);
+            fresnel_opts o = *opts;   // without the columns' scratch grids
+            o.fft_split_above = INT_MAX;
+            return plan_scattered_batch(problems, n, tol, &o, stream, out_plan);
         }
         p->subs.push_back(reinterpret_cast<Plan*>(h));
         p->N += p->subs.back()->N;

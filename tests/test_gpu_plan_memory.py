@@ -41,3 +41,39 @@ def test_held_memory_is_reported_and_small_plans_hold_little(kind):
     assert held <= 1.05 * reported + 4 * MB
     # at most as much again in the slabs as the tables in them, and one slab more
     assert plans[0].info()["device_bytes"] <= 2 * exact + (64 << 10)
+
+
+def test_a_plan_that_fits_without_its_scratch_grid_is_not_refused():
+    # FP32 scattered plans put columns above 2,400 points through a scratch grid
+    # of the FFT grid's size; with room for the plan but not for it, they take
+    # single passes.  The rest of the memory is taken by one tensor
+    from paper_2010_05978_gb300 import BatchPlan, Plan
+    g = W.rng(14, 0)
+    n, M = 300, 400
+    x, y, w = g.uniform(-1, 1, n), g.uniform(-1, 1, n), g.uniform(0.5, 1.5, n) / n
+    fam = {"kind": "nodes", "x": x, "y": y, "w": w}
+    t = torch.tensor(g.uniform(-1.5, 1.5, (M, 2)), device="cuda")
+    box = (-1.5, 1.5, -1.5, 1.5)
+    one = lambda **kw: Plan([fam], 0.0035, 1.0, 1e-6, box=box, **kw)
+    two = lambda **kw: BatchPlan([{"families": [fam], "lam": 0.0035, "z": 1.0}] * 2, 1e-6, box=box, **kw)
+    run = {one: lambda p: p.eval(t), two: lambda p: p.eval(torch.cat([t, t]), [M, M])}
+    for make in (one, two):
+        p = make(fft_split_above=1 << 30)
+        single, ref = p.info()["device_bytes"], run[make](p)
+        p.close()
+        p = make()
+        split = p.info()["device_bytes"]
+        assert float((run[make](p) - ref).norm() / ref.norm()) <= 2e-6
+        p.close()
+        assert split > single + 100 * MB
+        torch.cuda.empty_cache()
+        hog = torch.empty(_free() - (single + split) // 2, dtype=torch.uint8, device="cuda")
+        try:
+            p = make()
+            assert p.info()["device_bytes"] < single + 8 * MB
+            out = run[make](p)
+            p.close()
+        finally:
+            del hog
+            torch.cuda.empty_cache()
+        assert float((out - ref).norm() / ref.norm()) <= 2e-6
