@@ -1728,9 +1728,18 @@ fresnel_status adjoint_grid(Plan* p, const void* d_gamma) {
     if (!p->adj_in) FRES_TRY(dalloc(p, &p->adj_in, cs * (size_t)p->n1 * p->n2 * p->B));
     if (!p->adj_rows) FRES_TRY(dalloc(p, &p->adj_rows, cs * (size_t)p->n2 * p->nf1 * p->B));
     if (!p->contrib) FRES_TRY(dalloc(p, (void**)&p->contrib, sizeof(double) * p->N));
-    if (!p->d2.stw) {
-        FRES_TRY(dalloc(p, &p->d2.stw, cs * p->d2.fp.ntw));
-        launch_stage_twiddles(p->d2.fp, p->d2.stw, sizeof(T) == 8, p->st);
+    // stage twiddles of the columns, which a direct column DFT has none of: kept,
+    // or under a memory cap (which need not have room for them) made each time
+    // in the forward transform's intermediate (nf2 n1 >= ntw elements), free here
+    void* stw = p->d2.stw;
+    if (!stw) {
+        if (p->opts.max_device_bytes > 0) {
+            stw = p->inter;
+        } else {
+            FRES_TRY(dalloc(p, &p->d2.stw, cs * p->d2.fp.ntw));
+            stw = p->d2.stw;
+        }
+        launch_stage_twiddles(p->d2.fp, stw, sizeof(T) == 8, p->st);
     }
     launch_adj_prologue<T>(d_gamma, p->ax, p->ay, p->adj_in, p->n1, p->n2, p->B,
                            p->output == FRESNEL_OCCULTER, p->st);
@@ -1752,7 +1761,7 @@ fresnel_status adjoint_grid(Plan* p, const void* d_gamma) {
     ca.in_len = p->n2;
     ca.centered_in = 1;
     ca.out_len = p->nf2;
-    ca.twiddle = p->d2.stw;
+    ca.twiddle = stw;
     ca.out_is_final = 0;
     ca.batch = p->B;
     ca.in_bstride = (long long)p->n2 * p->nf1;

@@ -77,3 +77,29 @@ def test_a_plan_that_fits_without_its_scratch_grid_is_not_refused():
             del hog
             torch.cuda.empty_cache()
         assert float((out - ref).norm() / ref.norm()) <= 2e-6
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_a_capped_gradient_takes_only_its_own_arrays(prec):
+    # a starshade on a few cells (direct column DFT, which has no stage
+    # twiddles); a cap with room for the adjoint's two grids and the nodes'
+    # contributions is enough
+    from paper_2010_05978_gb300 import Plan
+    _, probs, grid, _ = W.spline_starshade("c4", n_coef=20, lams=(600e-9,), ngrid=64)
+    q = probs[0]
+    make = lambda cap: Plan([q["family"]], q["lam"], q["z"], 1e-6, precision=prec, output="occulter",
+                            grid=grid, max_device_bytes=cap)
+    p = make(1 << 40)
+    u = p.eval()
+    info, cs = p.info(), 8 if prec == "fp32" else 16
+    own = cs * 64 * 64 + cs * 64 * info["nf1"] + 8 * info["n_nodes"]
+    rest = 8 * 8   # where the family's gradient lies, and its number
+    g = p.grad_profile(u)
+    assert p.info()["device_bytes"] - info["device_bytes"] <= own + rest
+    p = make(info["device_bytes"] + own + rest)
+    got = p.grad_profile(p.eval())
+    again = p.grad_profile(p.eval())
+    ref = make(0)
+    ref = ref.grad_profile(ref.eval())
+    for v in (g, got, again):   # gradients repeat as their fields do
+        assert float((v - ref).norm() / ref.norm()) <= (2e-5 if prec == "fp32" else 1e-11)
