@@ -1208,6 +1208,10 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
             d->big = true;
             d->fpa = make_fft_plan(d->fa, dbl);
             d->fpb = make_fft_plan(d->fb, dbl);
+        } else if (fft_supported(d->n, dbl)) {
+            // fft_split_above below a length without a split into two passes of
+            // two stages each (50 is the one that a plan can have): one pass
+            d->fp = make_fft_plan(d->n, dbl);
         } else {
             return fres_fail(FRESNEL_ERR_UNSUPPORTED, "FFT length " + std::to_string(d->n) +
                                                           " has no supported split");
