@@ -404,7 +404,8 @@ typedef struct {
     int tile_x, tile_y;     /* spreading tile */
     long long device_bytes; /* device memory the plan holds */
     int launches_per_eval;  /* kernels launched by one fresnel_eval */
-    int split_tiles;        /* spreading tiles whose records are split over several work items */
+    int split_tiles;        /* spreading tiles whose records are split over several work items
+                               (0 for plans that spread by column strips) */
     int max_tile_records;   /* node records of the fullest spreading tile */
     int t3_binning;         /* FP32 SCATTERED plans: 1 binned interpolation, -1 direct
                                gathers, 0 chosen per evaluation (fresnel_opts.t3_binning,

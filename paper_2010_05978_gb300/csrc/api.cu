@@ -2166,7 +2166,7 @@ fresnel_status fresnel_get_info(fresnel_plan_t plan, fresnel_info* info) {
         info->device_bytes = bytes;
         info->launches_per_eval = launches;
         for (size_t i = 1; i < p->subs.size(); ++i) {
-            info->split_tiles += p->subs[i]->max_split;
+            info->split_tiles += p->subs[i]->strips ? 0 : p->subs[i]->max_split;
             info->max_tile_records = std::max(info->max_tile_records, p->subs[i]->det_tmax);
             info->live_tile_rows += (int)std::min<long long>(p->subs[i]->live_rows_total, INT_MAX);
         }
@@ -2188,7 +2188,7 @@ fresnel_status fresnel_get_info(fresnel_plan_t plan, fresnel_info* info) {
     if (p->opts.recompute_nodes) nl += 3;   // nodes, scan, scatter
     if (p->opts.deterministic) nl += 2;      // strengths' maxima, split tiles' conversion
     info->launches_per_eval = p->last_launches > 0 ? p->last_launches : nl;
-    info->split_tiles = p->max_split;
+    info->split_tiles = p->strips ? 0 : p->max_split;
     info->max_tile_records = p->det_tmax;
     info->t3_binning = p->opts.t3_binning;
     info->live_tile_rows = (int)std::min<long long>(p->live_rows_total, INT_MAX);

@@ -103,3 +103,12 @@ def test_a_capped_gradient_takes_only_its_own_arrays(prec):
     ref = ref.grad_profile(ref.eval())
     for v in (g, got, again):   # gradients repeat as their fields do
         assert float((v - ref).norm() / ref.norm()) <= (2e-5 if prec == "fp32" else 1e-11)
+
+
+def test_split_tiles_are_those_that_the_plan_splits():
+    from paper_2010_05978_gb300 import Plan
+    fam = W.fourier_family([1.0, 0.0, 0.0], 64, 16, 64)
+    make = lambda **kw: Plan([fam], 0.1, 1.0, 1e-6, grid=W.grid_spec(100, 100, 0.03), **kw)
+    assert make().info()["split_tiles"] == 0                    # by column strips
+    assert make(max_spin=1 << 22).info()["split_tiles"] > 0     # by tiles
+    assert make(deterministic=True).info()["split_tiles"] > 0
