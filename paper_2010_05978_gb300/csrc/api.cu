@@ -520,13 +520,11 @@ void ev_record(Plan* p, const char* name) {
 }
 
 template <typename T>
-fresnel_status run_nodes(Plan* p, double* dx, double* dy, double* dw) {
+fresnel_status run_nodes(Plan* p) {
     if (p->strips)
-        launch_nodes_strips<T>(p->ft, p->node_blocks, (NodeRec<T>*)p->rec, p->ss, dx, dy, dw,
-                               p->status, p->st);
+        launch_nodes_strips<T>(p->ft, p->node_blocks, (NodeRec<T>*)p->rec, p->ss, p->status, p->st);
     else
-        launch_nodes<T>(p->ft, p->node_blocks, (NodeRec<T>*)p->rec, p->counts, dx, dy, dw,
-                        p->status, p->st);
+        launch_nodes<T>(p->ft, p->node_blocks, (NodeRec<T>*)p->rec, p->counts, p->status, p->st);
     p->launches++;
     return FRESNEL_OK;
 }
@@ -676,7 +674,7 @@ fresnel_status eval_impl(Plan* p, const double* d_targets, long long M, void* d_
         FRES_CK(cudaEventRecord(p->ev_sorted, p->sort_st));
     }
     if (p->opts.recompute_nodes || !p->nodes_ready) {
-        FRES_TRY(run_nodes<T>(p, nullptr, nullptr, nullptr));
+        FRES_TRY(run_nodes<T>(p));
         ev_record(p, "nodes_chirp_count");
         FRES_TRY(run_sort<T>(p));
         ev_record(p, "scatter");
@@ -1419,7 +1417,7 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
     FRES_TRY(dalloc(p, (void**)&p->work, 2 * sizeof(int)));
     FRES_CK(cudaMemsetAsync(p->counts, 0, sizeof(int) * tt, p->st));
     FRES_CK(cudaMemsetAsync(p->work, 0, 2 * sizeof(int), p->st));
-    FRES_TRY(run_nodes<T>(p, nullptr, nullptr, nullptr));
+    FRES_TRY(run_nodes<T>(p));
     std::vector<int> hc(tt);
     FRES_CK(cudaMemcpyAsync(hc.data(), p->counts, sizeof(int) * tt, cudaMemcpyDeviceToHost, p->st));
     FRES_CK(cudaStreamSynchronize(p->st));
@@ -1586,7 +1584,7 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
                                 cudaMemcpyHostToDevice, p->st));
     }
     if (p->strips) {
-        FRES_TRY(run_nodes<T>(p, nullptr, nullptr, nullptr));   // the records under their keys
+        FRES_TRY(run_nodes<T>(p));   // the records under their keys
     } else {
         int* d_sc = nullptr;
         int* d_pl = nullptr;
@@ -2201,15 +2199,7 @@ fresnel_status fresnel_get_nodes(fresnel_plan_t plan, double* d_x, double* d_y, 
     if (!d_x || !d_y || !d_w) return fres_fail(FRESNEL_ERR_ARG, "node output arrays are NULL");
     if (!p->subs.empty())
         return fres_fail(FRESNEL_ERR_ARG, "scattered-target batch: nodes are per sub-plan");
-    // Regenerates the nodes (and, harmlessly, the unsorted records and counts),
-    // then re-runs the scan so the counts are reset and the cached sort stays valid.
-    if (p->prec == FRESNEL_FP64) {
-        FRES_TRY(run_nodes<double>(p, d_x, d_y, d_w));
-        FRES_TRY(run_sort<double>(p));
-    } else {
-        FRES_TRY(run_nodes<float>(p, d_x, d_y, d_w));
-        FRES_TRY(run_sort<float>(p));
-    }
+    launch_node_xyw(p->ft, p->node_blocks, d_x, d_y, d_w, p->st);
     FRES_CK(cudaGetLastError());
     return read_status(p);
 }

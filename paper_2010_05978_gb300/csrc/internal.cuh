@@ -363,11 +363,14 @@ void launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cuda
 // k_nodes.cu
 void launch_gauss_legendre(int n, double* t01, double* w01, cudaStream_t st);
 void launch_boundary(const FamilyDev& f, const ChirpParams& cp, cudaStream_t st);
-// All families of a plan in one launch: records, tile counts (keys offset by
-// each problem's tile_base) and, when dx != NULL, the FP64 nodes.
+// All families of a plan in one launch: records and tile counts (keys offset by
+// each problem's tile_base).
 template <typename T>
-void launch_nodes(const FamTable& ft, int nblocks, NodeRec<T>* rec, int* counts, double* dx,
-                  double* dy, double* dw, unsigned* status, cudaStream_t st);
+void launch_nodes(const FamTable& ft, int nblocks, NodeRec<T>* rec, int* counts, unsigned* status,
+                  cudaStream_t st);
+// the FP64 nodes alone
+void launch_node_xyw(const FamTable& ft, int nblocks, double* dx, double* dy, double* dw,
+                     cudaStream_t st);
 template <typename T>
 void launch_scatter_fams(const FamTable& ft, int nblocks, const NodeRec<T>* rec, int* cursor,
                          NodeRec<T>* sorted, long long cap, unsigned* status, cudaStream_t st);
@@ -375,7 +378,7 @@ void launch_scatter_fams(const FamTable& ft, int nblocks, const NodeRec<T>* rec,
 // starts and the scatter of the n records.
 template <typename T>
 void launch_nodes_strips(const FamTable& ft, int nblocks, NodeRec<T>* rec, const StripSort& ss,
-                         double* dx, double* dy, double* dw, unsigned* status, cudaStream_t st);
+                         unsigned* status, cudaStream_t st);
 void launch_strip_starts(const StripSort& ss, cudaStream_t st);
 template <typename T>
 void launch_scatter_strips(long long n, const NodeRec<T>* rec, const StripSort& ss,

@@ -448,11 +448,9 @@ __device__ __forceinline__ void node_tri_df(const FamilyDev& f, const ChirpParam
     finish_df(v1, v2, cre, cim, cp, rec + f.offset + j, status, cell);
 }
 
-template <typename T>
-__device__ __forceinline__ void node_generic(const FamilyDev& f, const ChirpParams& cp, long long j,
-                                             NodeRec<T>* rec, double* dx, double* dy, double* dw,
-                                             unsigned* status, int2& cell, const ScreenDev& scr) {
-    double x, y, w;
+// Position and weight of node j in FP64.
+__device__ __forceinline__ void node_xyw(const FamilyDev& f, long long j, double& x, double& y,
+                                         double& w) {
     if (f.kind == FRESNEL_FAMILY_NODES) {
         x = f.params[j];
         y = f.params[f.n_nodes + j];
@@ -491,12 +489,15 @@ __device__ __forceinline__ void node_generic(const FamilyDev& f, const ChirpPara
         y = f.cy + a * f.by[i];
         w = f.gl_m_aw[l] * f.bc[i];
     }
-    long long g = f.offset + j;
-    if (dx) {
-        dx[g] = x;
-        dy[g] = y;
-        dw[g] = w;
-    }
+}
+
+template <typename T>
+__device__ __forceinline__ void node_generic(const FamilyDev& f, const ChirpParams& cp, long long j,
+                                             NodeRec<T>* rec, unsigned* status, int2& cell,
+                                             const ScreenDev& scr) {
+    double x, y, w;
+    node_xyw(f, j, x, y, w);
+    const long long g = f.offset + j;
     double ph = reduce_phase(cp.kq * (x * x + y * y) - cp.a1 * x - cp.a2 * y + cp.a0);
     NodeRec<T> r;
     if (sizeof(T) == 8) {
@@ -597,12 +598,13 @@ __device__ __forceinline__ void load_family(const FamTable& ft, FamSmem& sm) {
 // FP32 fast mode runs the dilation families in the double-float spoke form
 // (no FP64 per node); FP64 per node otherwise.  One launch covers every
 // family of every problem of the plan.
-// STRIPS: counts and ranks under the strip keys of `ss`; else counts of every
-// tile that the support touches.
-template <typename T, bool STRIPS>
+// Counts of every tile that the support touches, or, where ss has its map of
+// the tiles (ss.live), counts and ranks under its strip keys: one kernel for
+// the plan's count, from which that map is made, and for the evaluations, so
+// that a node at a tile's edge falls on the same side in both.
+template <typename T>
 __global__ void __launch_bounds__(kNodeThreads)
-k_nodes(FamTable ft, NodeRec<T>* rec, int* counts, StripSort ss, double* dx, double* dy,
-        double* dw, unsigned* status) {
+k_nodes(FamTable ft, NodeRec<T>* rec, int* counts, StripSort ss, unsigned* status) {
     __shared__ __align__(16) FamSmem sm;
     kernel_begin();
     load_family(ft, sm);
@@ -611,21 +613,21 @@ k_nodes(FamTable ft, NodeRec<T>* rec, int* counts, StripSort ss, double* dx, dou
     int2 cell = make_int2(0, 0);
     if (j < f.n_nodes) {
         if constexpr (sizeof(T) == 4) {
-            if (f.spoke && !dx)
+            if (f.spoke)
                 node_df(f, sm.cp, j, reinterpret_cast<NodeRec<float>*>(rec), status, cell, ft.scr);
-            else if (f.ptab && !dx)
+            else if (f.ptab)
                 node_petal_df(f, sm.cp, j, reinterpret_cast<NodeRec<float>*>(rec), status, cell,
                               ft.scr);
-            else if (f.tdf && !dx)
+            else if (f.tdf)
                 node_tri_df(f, sm.cp, j, reinterpret_cast<NodeRec<float>*>(rec), status, cell,
                             ft.scr);
             else
-                node_generic<T>(f, sm.cp, j, rec, dx, dy, dw, status, cell, ft.scr);
+                node_generic<T>(f, sm.cp, j, rec, status, cell, ft.scr);
         } else {
-            node_generic<T>(f, sm.cp, j, rec, dx, dy, dw, status, cell, ft.scr);
+            node_generic<T>(f, sm.cp, j, rec, status, cell, ft.scr);
         }
     }
-    if constexpr (STRIPS) {
+    if (ss.live) {
         int key = -1;
         if (j < f.n_nodes) {
             const int lt = ss.live[sm.cp.tile_base + (cell.y / kTile) * sm.cp.ntx + cell.x / kTile];
@@ -640,6 +642,21 @@ k_nodes(FamTable ft, NodeRec<T>* rec, int* counts, StripSort ss, double* dx, dou
 #pragma unroll
         for (int k = 0; k < 4; ++k) agg_count(key[k], counts);
     }
+}
+
+// The nodes themselves (fresnel_get_nodes): no record, count or rank is touched.
+__global__ void __launch_bounds__(kNodeThreads)
+k_node_xyw(FamTable ft, double* __restrict__ dx, double* __restrict__ dy, double* __restrict__ dw) {
+    __shared__ __align__(16) FamSmem sm;
+    load_family(ft, sm);
+    const long long j = (long long)(blockIdx.x - sm.b0) * blockDim.x + threadIdx.x;
+    if (j >= sm.f.n_nodes) return;
+    double x, y, w;
+    node_xyw(sm.f, j, x, y, w);
+    const long long g = sm.f.offset + j;
+    dx[g] = x;
+    dy[g] = y;
+    dw[g] = w;
 }
 
 // Key starts of a strip-sorted plan: a block scans 1024 consecutive keys'
@@ -1162,28 +1179,30 @@ void launch_boundary(const FamilyDev& f, const ChirpParams& cp, cudaStream_t st)
 }
 
 template <typename T>
-void launch_nodes(const FamTable& ft, int nblocks, NodeRec<T>* rec, int* counts, double* dx,
-                  double* dy, double* dw, unsigned* status, cudaStream_t st) {
+void launch_nodes(const FamTable& ft, int nblocks, NodeRec<T>* rec, int* counts, unsigned* status,
+                  cudaStream_t st) {
     if (nblocks <= 0) return;
-    k_nodes<T, false><<<nblocks, kNodeThreads, 0, st>>>(ft, rec, counts, StripSort{}, dx, dy, dw,
-                                                        status);
+    k_nodes<T><<<nblocks, kNodeThreads, 0, st>>>(ft, rec, counts, StripSort{}, status);
 }
-template void launch_nodes<float>(const FamTable&, int, NodeRec<float>*, int*, double*, double*,
-                                  double*, unsigned*, cudaStream_t);
-template void launch_nodes<double>(const FamTable&, int, NodeRec<double>*, int*, double*,
-                                   double*, double*, unsigned*, cudaStream_t);
+template void launch_nodes<float>(const FamTable&, int, NodeRec<float>*, int*, unsigned*, cudaStream_t);
+template void launch_nodes<double>(const FamTable&, int, NodeRec<double>*, int*, unsigned*,
+                                   cudaStream_t);
 
 template <typename T>
 void launch_nodes_strips(const FamTable& ft, int nblocks, NodeRec<T>* rec, const StripSort& ss,
-                         double* dx, double* dy, double* dw, unsigned* status, cudaStream_t st) {
+                         unsigned* status, cudaStream_t st) {
     if (nblocks <= 0) return;
-    launch_after(k_nodes<T, true>, nblocks, kNodeThreads, 0, st, ft, rec, nullptr, ss, dx, dy, dw,
-                 status);
+    launch_after(k_nodes<T>, nblocks, kNodeThreads, 0, st, ft, rec, nullptr, ss, status);
 }
 template void launch_nodes_strips<float>(const FamTable&, int, NodeRec<float>*, const StripSort&,
-                                         double*, double*, double*, unsigned*, cudaStream_t);
+                                         unsigned*, cudaStream_t);
 template void launch_nodes_strips<double>(const FamTable&, int, NodeRec<double>*, const StripSort&,
-                                          double*, double*, double*, unsigned*, cudaStream_t);
+                                          unsigned*, cudaStream_t);
+
+void launch_node_xyw(const FamTable& ft, int nblocks, double* dx, double* dy, double* dw,
+                     cudaStream_t st) {
+    if (nblocks > 0) k_node_xyw<<<nblocks, kNodeThreads, 0, st>>>(ft, dx, dy, dw);
+}
 
 void launch_strip_starts(const StripSort& ss, cudaStream_t st) {
     if (ss.nkeys > 0) launch_after(k_strip_starts, nblk(ss.nkeys, 1024), 256, 0, st, ss);
