@@ -1533,14 +1533,22 @@ fresnel_status build_plan(Plan* p, const fresnel_problem* problems) {
     // star FP32 spread 61 -> 25 us, FP64 at w = 13 1647 -> 627 us.  By
     // tiles where that form is asked for: exact fixed-point sums
     // (deterministic), a bounded ready-flag wait (max_spin set); where rows or
-    // keys would overflow 32 bits; and where a memory cap is set that the
-    // strip sort's arrays could miss though the tile sort's fit.
+    // keys would overflow 32 bits; where a memory cap is set that the strip
+    // sort's arrays could miss though the tile sort's fit; and for few records,
+    // which leave the strips too few warps while each tile has a block (us per
+    // call, strips / tiles, nodes all over a grid of 256^2: FP64 300 86.6 / 51.0,
+    // 2000 80.7 / 57.7, 4000 77.9 / 82.4; FP32 300 32.7 / 26.8, 4000 27.1 / 30.2;
+    // a star's: FP64 256 80.3 / 56.9, 1152 76.9 / 82.4; FP32 256 29.0 / 26.9, 640
+    // 25.0 / 28.5; regenerated FP32 nodes 300 42.2 / 47.3: the strip sort is the
+    // faster one).
     const long long nkeys = n_live * kStripKeys;
     {
+        const long long from = dbl ? (p->strip_merge ? 3500 : 800)
+                                   : (p->opts.recompute_nodes ? 0 : (p->strip_merge ? 4000 : 500));
         const long long rs = (long long)p->rsize();
         const long long by_tiles = rs * p->n_records + (long long)sizeof(Chunk) * p->max_chunks;
         const long long by_strips = (rs + 4) * p->N + 8 * nkeys + 4 * tt + 64;
-        p->strips = !p->opts.deterministic && p->opts.max_spin == 0 &&
+        p->strips = !p->opts.deterministic && p->opts.max_spin == 0 && p->N >= from &&
                     (long long)p->B * p->nf2 < (1LL << 31) && nkeys < (1LL << 31) &&
                     !(p->opts.max_device_bytes > 0 && by_strips > by_tiles);
     }

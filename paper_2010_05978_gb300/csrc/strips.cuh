@@ -320,6 +320,11 @@ k_spread_strips_f32(const NodeRec<float>* __restrict__ sorted, long long n, int 
 }
 
 // ------------------------------------------------------------------ FP64
+// By the bits: a comparison takes the FP64 pipe as long as a multiply-add.
+__device__ __forceinline__ bool nonzero(double2 v) {
+    return ((__double_as_longlong(v.x) | __double_as_longlong(v.y)) << 1) != 0;
+}
+
 template <int W>
 struct StripSmemD {
     static constexpr int COLS = W + 7;
@@ -358,19 +363,21 @@ k_spread_strips_f64(const NodeRec<double>* __restrict__ sorted, long long n, int
         d = d < W ? d : W;
         int x = cur_a * 8 + lane;
         if (x >= nf1) x -= nf1;
-        for (int o = 0; o < d; ++o) {
-            int y = cur_b + o;
-            double2* cell = win + (y & 15) * COLS + lane;
-            if (y >= yend) y -= nf2;
-            if (lane < COLS) {
-                const double2 v = *cell;
-                if (v.x != 0.0 || v.y != 0.0) {
-                    *cell = make_double2(0.0, 0.0);
-                    double2* g = grid + (long long)y * nf1 + x;
-                    atomicAdd(&g->x, v.x);
-                    atomicAdd(&g->y, v.y);
+        for (int o = 0; o < d; o += 2) {
+            double2 v[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                v[i] = o + i < d && lane < COLS ? win[((cur_b + o + i) & 15) * COLS + lane]
+                                                : make_double2(0.0, 0.0);
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                if (nonzero(v[i])) {
+                    const int y = cur_b + o + i;
+                    win[(y & 15) * COLS + lane] = make_double2(0.0, 0.0);
+                    double2* g = grid + (long long)(y >= yend ? y - nf2 : y) * nf1 + x;
+                    atomicAdd(&g->x, v[i].x);
+                    atomicAdd(&g->y, v[i].y);
                 }
-            }
         }
         __syncwarp();
     };
@@ -433,7 +440,7 @@ k_spread_strips_f64(const NodeRec<double>* __restrict__ sorted, long long n, int
         all, make_int2(cur_a, cur_b), nf1, nf2,
         [](const StripSmemD<W>& w, int y, int x) { return w.win[(y & 15) * COLS + x]; },
         [&](int x, int y, double2 v) {
-            if (v.x == 0.0 && v.y == 0.0) return;
+            if (!nonzero(v)) return;
             double2* g = grid + (long long)y * nf1 + x;
             atomicAdd(&g->x, v.x);
             atomicAdd(&g->y, v.y);

@@ -122,7 +122,7 @@ def test_blocks_that_merge_their_rows(prec, w):
     # them on 40 points (runs of warps on one strip), record counts at the
     # edges of a batch, of a block and of the widest blocks
     from paper_2010_05978_gb300 import Plan
-    for n in (1, 33, 511, 513, 1025, 30000, 117000):
+    for n in (1, 33, 511, 513, 1025, 4096, 4607, 4609, 4641, 30000, 117000):
         g = W.rng(12, 100 * n + w)
         x, y = g.uniform(-1, 1, n), g.uniform(-1, 1, n)
         k = g.integers(0, min(40, n), n // 2)
