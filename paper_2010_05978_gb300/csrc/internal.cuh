@@ -329,6 +329,12 @@ struct ScanLayout {
 };
 constexpr int kMaxTileRows = 256;   // nf2 <= 8192
 
+// FP64 by the bits: a comparison takes the FP64 pipe as long as a multiply-add.
+__device__ __forceinline__ bool nonzero(float2 v) { return v.x != 0.0f || v.y != 0.0f; }
+__device__ __forceinline__ bool nonzero(double2 v) {
+    return ((__double_as_longlong(v.x) | __double_as_longlong(v.y)) << 1) != 0;
+}
+
 // Programmatic dependent launch: a kernel launched with launch_after may be
 // scheduled while the kernel before it in the stream is still finishing.  It
 // first calls kernel_begin() in every thread of every block, before any memory

@@ -451,7 +451,7 @@ k_fft_rows(FftPlan fp, RowPassArgs a, int lines, int tr) {
     batched<C>(
         pl, a.in_len, [&](int i) { return in[i]; },
         [&](int i, C v) {
-            if (a.clear_in && (v.x != (T)0 || v.y != (T)0)) in[i] = Ops<T>::mk(0, 0);
+            if (a.clear_in && nonzero(v)) in[i] = Ops<T>::mk(0, 0);
             if (a.centered_in) v = Ops<T>::scale(v, rowf * (dcol ? __ldg(&dcol[i]) : (T)1));
             S[pl.c + pad(in_natural(i, a.in_len, n, a.centered_in))] = v;
         });
@@ -529,7 +529,7 @@ k_fft_cols(FftPlan fp, ColPassArgs a, int ls) {
             [&](int ea, C v) {
                 const int i = src(ea);
                 if (i < 0) return v;
-                if (a.clear_in && (v.x != (T)0 || v.y != (T)0)) in[i] = O::mk(0, 0);
+                if (a.clear_in && nonzero(v)) in[i] = O::mk(0, 0);
                 if (a.centered_in) v = O::scale(v, rowf * (dcol ? __ldg(&dcol[i]) : (T)1));
                 return v;
             });
@@ -717,7 +717,13 @@ void launch_cols_mode(const FftPlan& fp, const ColPassArgs& a, cudaStream_t st) 
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(k_fft_cols<T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
-    launch_after(k_fft_cols<T, MODE>, blocks, threads, smem, st, fp, a, ls);
+    // FP64 plainly where the blocks fill the SMs: placed early, by the room that
+    // the row pass leaves, they load them unevenly (800-point columns of a star's
+    // field 139 -> 121 us a call, its gradient at 512 points 614 -> 602)
+    if (sizeof(T) == 8 && blocks >= 152)
+        k_fft_cols<T, MODE><<<blocks, threads, smem, st>>>(fp, a, ls);
+    else
+        launch_after(k_fft_cols<T, MODE>, blocks, threads, smem, st, fp, a, ls);
 }
 
 // FP32 column passes of square type-3 grids, start (two buffers, radix-16/8/4/

@@ -320,11 +320,6 @@ k_spread_strips_f32(const NodeRec<float>* __restrict__ sorted, long long n, int 
 }
 
 // ------------------------------------------------------------------ FP64
-// By the bits: a comparison takes the FP64 pipe as long as a multiply-add.
-__device__ __forceinline__ bool nonzero(double2 v) {
-    return ((__double_as_longlong(v.x) | __double_as_longlong(v.y)) << 1) != 0;
-}
-
 template <int W>
 struct StripSmemD {
     static constexpr int COLS = W + 7;
