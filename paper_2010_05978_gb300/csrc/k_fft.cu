@@ -448,17 +448,39 @@ k_fft_rows(FftPlan fp, RowPassArgs a, int lines, int tr) {
     C* in = (C*)a.in + (long long)row * a.in_stride;
     C* out = (C*)a.out + (long long)row * a.out_stride;
     const T rowf = a.deconv_row ? ((const T*)a.deconv_row)[row] : (T)1;
-    batched<C>(
-        pl, a.in_len, [&](int i) { return in[i]; },
-        [&](int i, C v) {
-            if (a.clear_in && nonzero(v)) in[i] = Ops<T>::mk(0, 0);
-            if (a.centered_in) v = Ops<T>::scale(v, rowf * (dcol ? __ldg(&dcol[i]) : (T)1));
-            S[pl.c + pad(in_natural(i, a.in_len, n, a.centered_in))] = v;
-        });
-    zero_rest(S, pl, a.in_len, n, a.centered_in);
-    __syncthreads();
-    fft_line<T>(S, fp, pl, tw);
-    for (int kp = pl.t; kp < a.out_len; kp += tr) out[kp] = S[pl.c + pad(out_natural(kp, a.out_len, n))];
+    auto use = [&](int i, C v) {   // input i, read as v
+        if (a.clear_in && nonzero(v)) in[i] = Ops<T>::mk(0, 0);
+        if (a.centered_in) v = Ops<T>::scale(v, rowf * (dcol ? __ldg(&dcol[i]) : (T)1));
+        return v;
+    };
+    if constexpr (sizeof(T) == 8) {
+        // few radices, so little code: reads and stores in the first and last
+        // stages (us, from start over short loops to fused: 500 x 500 nodes' rows
+        // of 1024 33.4, 37.5, 35.5; of 2048 66.2, 70.3, 66.2)
+        auto input = make_input(
+            [&](int e) {
+                const int i = in_src(e, a.in_len, n, a.centered_in);
+                return i < 0 ? Ops<T>::mk(0, 0) : in[i];
+            },
+            [&](int e, C v) {
+                const int i = in_src(e, a.in_len, n, a.centered_in);
+                return i < 0 ? v : use(i, v);
+            });
+        auto store = [&](int k, C v) {
+            const int kp = out_slot(k, a.out_len, n);
+            if (kp >= 0) out[kp] = v;
+        };
+        fft_fused<T>(S, fp, pl, pl, tw, input, store);
+    } else {
+        batched<C>(
+            pl, a.in_len, [&](int i) { return in[i]; },
+            [&](int i, C v) { S[pl.c + pad(in_natural(i, a.in_len, n, a.centered_in))] = use(i, v); });
+        zero_rest(S, pl, a.in_len, n, a.centered_in);
+        __syncthreads();
+        fft_line<T>(S, fp, pl, tw);
+        for (int kp = pl.t; kp < a.out_len; kp += tr)
+            out[kp] = S[pl.c + pad(out_natural(kp, a.out_len, n))];
+    }
 }
 
 // Columns: a block takes 2^ls adjacent columns.
