@@ -172,7 +172,9 @@ typedef struct {
      * per pass through an intermediate buffer) instead of one shared-memory
      * pass; 0 = when one pass does not fit in shared memory (lengths above
      * ~13,600 in FP32, ~6,800 in FP64), and for FP32 SCATTERED plans without
-     * a memory cap also columns above 2,400, where four steps are faster.
+     * a memory cap also columns above 2,400, where four steps are faster (one
+     * pass where their buffer does not fit).  A length without a split into
+     * two passes stays one.
      * Batched plans and profile gradients need single-pass lengths. */
     int fft_split_above;
     /* 1: measure before committing to a configuration.  FP64 with automatic
@@ -212,9 +214,9 @@ typedef struct {
      * chunks of a tile that holds more records than one work item takes wait,
      * before adding into the tile, for the flag with which the tile's first
      * chunk reports having cleared it.  0 (default): plans spread by column
-     * strips, where nothing waits (by tiles, with the built-in bound, only
-     * where a memory cap leaves no room for the strip sort); any other value
-     * selects the tiles.  Polls per wait (~256 ns apart) before the
+     * strips, where nothing waits (by tiles, with the built-in bound, where a
+     * memory cap leaves no room for the strip sort and where a plan has few
+     * nodes, some hundreds to 4,000); any other value selects the tiles.  Polls per wait (~256 ns apart) before the
      * wait gives up, skips its addition and flags FRESNEL_ERR_TIMEOUT (read by
      * fresnel_check or a synchronous evaluation): 0 = the built-in 2^22
      * (about a second), > 0 = that many, < 0 = none at all (every such wait

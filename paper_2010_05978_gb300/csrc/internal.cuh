@@ -346,7 +346,7 @@ __device__ __forceinline__ bool nonzero(double2 v) {
 // 161 -> 155, sweep 144 -> 138, kite 33.0 -> 31.1).  The strip spreading is
 // launched plainly: its blocks take very different times, and placed early, by
 // the room that the earlier kernel leaves, they load the SMs unevenly (kite 34.3,
-// star grid 80.6).
+// star grid 80.6); so are FP64 column passes that fill the SMs (k_fft.cu).
 __device__ __forceinline__ void kernel_begin() {
     asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
 }

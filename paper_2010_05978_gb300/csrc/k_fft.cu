@@ -21,11 +21,11 @@
 // fewer stages (radices up to 16 with the composite 15, 12, 10 and 9, which
 // need no inner twiddles but 9's and 16's) and twiddles read consecutively from a table
 // per stage matter more than operations, and so does the code a block
-// runs once: in the single passes one body per radix serves every stage, with
-// the pruning, factors and epilogue in the short loops that fill and empty
+// runs once: in the FP32 single passes one body per radix serves every stage,
+// with the pruning, factors and epilogue in the short loops that fill and empty
 // the lines (fused into the first and last stages they made 33 KB of
 // straight-line code, whose fetching took up to half of a pass: 29 against 19
-// us cold for the star's 928 rows of 2048).  The four-step passes are short
+// us cold for the star's 928 rows of 2048; rows of 256 and 640 points 2 us more).  The four-step passes are short
 // transforms over gigabytes: there the code stays fetched, and they read and
 // store in their first and last stages (17,280^2 points: 3.6 against 4.8 ms).
 #include <algorithm>

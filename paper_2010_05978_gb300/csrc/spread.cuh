@@ -4,8 +4,9 @@
 // the first stage of the type-1 (Sec. 3.3) and type-3 (Sec. 3.2, eq. nufft3)
 // NUFFTs of arXiv:2010.05978 (the paper uses them as a library, FINUFFT).
 //
-// This is the tile form: deterministic plans, plans that set max_spin and the
-// standalone spreaders use it; other plans spread by strips (strips.cuh).
+// This is the tile form: deterministic plans, plans that set max_spin, plans of
+// few records, plans whose memory cap only its arrays meet and the standalone
+// spreaders use it; other plans spread by strips (strips.cuh).
 //
 // Owner-computes tiles: every 32 x 32 tile of the grid is produced by one
 // work item.  Nodes whose support straddles tiles were duplicated into each

@@ -46,7 +46,7 @@
 // FP64 (k_spread_strips_f64): the FP64 pipe (1/58 of the FP32 rate) bounds
 // it, so no multiply-add goes to padding: lanes walk the w x w support
 // (ceil(w^2 / 32) steps) on a private 16-row window in shared memory.  Star,
-// w = 13: 1649 -> 637 us; w = 10: 1016 -> 389 us.
+// w = 13: 1649 -> 609 us; w = 10: 1016 -> 392 us.
 #pragma once
 #include <algorithm>
 
