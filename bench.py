@@ -218,24 +218,20 @@ def rel_error(u, ref, tol, occulter=False):
 # Source files each measured kernel is built from (the DRAM traffic of an
 # ncu capture holds only while these are unchanged).
 KERNEL_SOURCES = {
-    "spread": ["spread.cuh", "k_spread_f32.cu", "internal.cuh"],
+    "spread": ["strips.cuh", "k_strips_f32.cu", "spread.cuh", "internal.cuh"],
     "interp": ["k_interp.cu", "spread.cuh", "dfloat.cuh", "internal.cuh"],
     "fft": ["k_fft.cu", "k_col_dft_tc.cu", "internal.cuh"],
     "nodes": ["k_nodes.cu", "dfloat.cuh", "internal.cuh"],
 }
 
-# Per launch, from one ncu capture of the named workload (sections
-# SpeedOfLight, MemoryWorkloadAnalysis, ComputeWorkloadAnalysis, Occupancy,
-# LaunchStats, SchedulerStats, WarpStateStats, InstructionStats): DRAM bytes
-# read + written (dram__bytes.sum.per_second x gpu__time_duration.sum), and the
-# SM-side utilisations (issue slots busy, LSU pipe, L1/TEX throughput, each a
-# fraction of its own peak), with the sha256 prefix of the kernel's sources
-# at the time of the capture.  A kernel whose sources changed since reports
-# traffic null.
-_CAP_STAR = "ncu capture of this workload (second warm-up step, every kernel)"
-_CAP_SWEEP = "ncu capture of this workload (second warm-up step)"
-_CAP_R1000 = "ncu capture of this workload at 3e7 targets (the spread does not depend on them)"
-_SHA_SPREAD, _SHA_FFT, _SHA_INTERP = "96e6910da872462a", "6c767b5c00f7c5ff", "6d7b1b741a45e8d0"
+# Per launch, from one ncu capture of the named workload: DRAM bytes read +
+# written (dram__bytes_read.sum + dram__bytes_write.sum) and the SM-side
+# utilisations (issue slots, LSU pipe, L1/TEX throughput, each a fraction of its
+# own peak), with the sha256 prefix of the kernel's sources at the time of the
+# capture.  A kernel whose sources changed since reports traffic null.
+_CAP_STAR = "ncu capture of this workload (third step, every kernel)"
+_CAP_SWEEP = "ncu capture of this workload (third step)"
+_SHA_SPREAD, _SHA_FFT, _SHA_INTERP = "a9c848d54bbaf453", "94c8d3055e21ee0b", "fb32c71246acce1f"
 
 
 def _cap(nbytes, issue, lsu, l1, sha, note):
@@ -245,21 +241,16 @@ def _cap(nbytes, issue, lsu, l1, sha, note):
 
 
 DRAM_TRAFFIC = {
-    ("star5_F100", "t1.spread"): _cap(18212608, 0.487, 0.408, 0.704, _SHA_SPREAD, _CAP_STAR),
-    ("star5_F100", "t3.spread"): _cap(19070208, 0.483, 0.413, 0.698, _SHA_SPREAD, _CAP_STAR),
-    ("star5_F100", "t1.fft_rows"): _cap(15313152, 0.273, 0.099, 0.495, _SHA_FFT, _CAP_STAR),
-    ("star5_F100", "t1.fft_cols_epilogue"): _cap(7558144, 0.230, 0.063, 0.266, _SHA_FFT,
-                                                 _CAP_STAR),
-    ("star5_F100", "t3.fft_rows"): _cap(6747392, 0.350, 0.126, 0.304, _SHA_FFT, _CAP_STAR),
-    ("star5_F100", "t3.fft_cols"): _cap(15152384, 0.361, 0.103, 0.455, _SHA_FFT, _CAP_STAR),
-    ("star5_F100", "t3.interp_epilogue"): _cap(21465344, 0.608, 0.350, 0.902, _SHA_INTERP,
-                                               _CAP_STAR),
-    ("hg24_sweep64", "spread"): _cap(23639579, 0.508, 0.430, 0.761, _SHA_SPREAD, _CAP_SWEEP),
-    ("hg24_sweep64", "fft_rows"): _cap(16898826, 0.308, 0.104, 0.420, _SHA_FFT, _CAP_SWEEP),
-    ("hg24_sweep64", "fft_cols_epilogue"): _cap(81341417, 0.393, 0.078, 0.627, _SHA_FFT,
-                                                _CAP_SWEEP),
-    ("randstar20_F1000", "spread"): _cap(826690109, 0.511, 0.431, 0.728, _SHA_SPREAD,
-                                         _CAP_R1000),
+    ("star5_F100", "t1.spread"): _cap(16301568, 0.712, 0.251, 0.659, _SHA_SPREAD, _CAP_STAR),
+    ("star5_F100", "t3.spread"): _cap(16143360, 0.706, 0.256, 0.659, _SHA_SPREAD, _CAP_STAR),
+    ("star5_F100", "t1.fft_rows"): _cap(15292160, 0.403, 0.169, 0.339, _SHA_FFT, _CAP_STAR),
+    ("star5_F100", "t1.fft_cols_epilogue"): _cap(7531776, 0.424, 0.139, 0.292, _SHA_FFT, _CAP_STAR),
+    ("star5_F100", "t3.fft_rows"): _cap(6730496, 0.423, 0.177, 0.389, _SHA_FFT, _CAP_STAR),
+    ("star5_F100", "t3.fft_cols"): _cap(13395456, 0.496, 0.161, 0.436, _SHA_FFT, _CAP_STAR),
+    ("star5_F100", "t3.interp_epilogue"): _cap(21479424, 0.516, 0.274, 0.849, _SHA_INTERP, _CAP_STAR),
+    ("hg24_sweep64", "spread"): _cap(23677440, 0.793, 0.289, 0.768, _SHA_SPREAD, _CAP_SWEEP),
+    ("hg24_sweep64", "fft_rows"): _cap(16862208, 0.452, 0.191, 0.362, _SHA_FFT, _CAP_SWEEP),
+    ("hg24_sweep64", "fft_cols_epilogue"): _cap(81243904, 0.388, 0.077, 0.622, _SHA_FFT, _CAP_SWEEP),
 }
 
 
