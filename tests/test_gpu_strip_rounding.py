@@ -9,7 +9,8 @@ field or gradient to which some ten (gradients: two) cells or modes contribute
 independently, so the logarithm of its root mean square over 8 repeats
 scatters by 1 / sqrt(2 * 8 * 10) = 0.08 (gradients 0.18) and a group of n
 quotients by sqrt(2 / n) times that; the bars lie four such deviations above 1
-(and 1.15 at least: a strip's rows close with one addition more than a tile)."""
+(and 1.15 at least: a strip's rows close with one addition more than a tile).
+20 repeats are taken, as a gradient's error may lie in one mode alone."""
 import numpy as np
 import pytest
 
@@ -18,7 +19,7 @@ import workloads as W
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
-REPEATS = 8
+REPEATS = 20
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -83,19 +84,23 @@ def test_wide_kernels_and_fp64(prec, opts, designs):
 @pytest.mark.parametrize("prec", ["fp32", "fp64"])
 def test_starshade_beside_a_disc_that_covers_the_grid(prec):
     from paper_2010_05978_gb300 import BatchPlan
-    _, probs, grid, _ = W.spline_starshade("c4", n_coef=60, lams=(600e-9,), ngrid=128)
-    s = probs[0]
-    disc = W.fourier_family([0.45 * s["lam"] * s["z"] / grid["h"], 0.0, 0.0], 200, 16, 100)
-    both = [{"families": [f], "lam": s["lam"], "z": s["z"]} for f in (disc, s["family"])]
 
-    def make(**kw):
-        p = BatchPlan(both, 1e-6, precision=prec, output="occulter", grid=grid, **kw)
-        u = p.eval()
-        return u[0], u[1], p.grad_profile(u * (2.0 / u.numel()))
+    def mixed(n, n_coef):
+        _, probs, grid, _ = W.spline_starshade("c4", n_coef=n_coef, lams=(600e-9,), ngrid=n)
+        s = probs[0]
+        disc = W.fourier_family([0.45 * s["lam"] * s["z"] / grid["h"], 0.0, 0.0], 200, 16, 100)
+        both = [{"families": [f], "lam": s["lam"], "z": s["z"]} for f in (disc, s["family"])]
 
-    q = _quotients(make)
-    _held(q[:2], 0.08)
-    _held(q[2:], 0.18)
+        def make(**kw):
+            p = BatchPlan(both, 1e-6, precision=prec, output="occulter", grid=grid, **kw)
+            u = p.eval()
+            return u[0], u[1], p.grad_profile(u * (2.0 / u.numel()))
+
+        return _quotients(make)
+
+    q = np.array([mixed(n, n_coef) for n, n_coef in ((128, 60), (128, 30), (100, 60), (112, 90))])
+    _held(q[:, :2].ravel(), 0.08)
+    _held(q[:, 2], 0.18)
 
 
 @pytest.mark.parametrize("prec", ["fp32", "fp64"])
